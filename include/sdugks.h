@@ -89,7 +89,10 @@ typedef struct sdugks_params {
     int32_t kernel;      /* SDUGKS_KERNEL_*                                        */
     int32_t tile_cells;  /* tiled kernel: cells per tile (16..128); Cartesian kernel (FP32,
                             bf16 and fp16 storage): 256, 224 or 128 for 16x16, 16x14 or 16x8 blocks;
-                            0 = chosen from the grid size (Cartesian) or 128 (tiled) */
+                            0 = chosen from the grid size (Cartesian) or 128 (tiled).  With
+                            plain loads, FP32 grids of many waves of blocks (about 430^2
+                            cells and up, no symmetry side) are stepped by marching warps
+                            instead; the blocks then run the diagnostic steps only */
     int32_t graph_steps; /* steps per captured CUDA graph in sdugks_step, 0 = auto, <0 = off */
     int32_t staging;     /* SDUGKS_STAGING_*; TMA requires the Cartesian kernel (else
                             INVALID_ARG).  A TMA copy that does not land within the wait
@@ -104,7 +107,7 @@ typedef struct sdugks_params {
 /* What a solver chose and holds (sdugks_solver_info). */
 typedef struct sdugks_info {
     int64_t n_cells, n_faces;     /* after periodic faces are merged pairwise          */
-    int64_t n_tiles;              /* CTAs per step                                     */
+    int64_t n_tiles;              /* tiles (blocks) of the grid: CTAs of a block or tile step */
     int64_t halo_cells;           /* summed over tiles (ring 1 + ring 2)               */
     int64_t steps_done;           /* steps since init / set_state                      */
     int64_t device_bytes;         /* device memory held by the solver                  */
@@ -310,12 +313,13 @@ void sdugks_autotune_clear(void);
 
 /* ---- batched solves ----------------------------------------------------------- */
 /* Many independent uniform-grid solves (cavities, channels) of different sizes and
- * Reynolds numbers advanced together: every step is one launch over the (instance,
- * 16x8 block) work list of all instances, one CTA per item (or, if the autotuner
- * prefers it, a fixed grid of CTAs walking the list), with the S-DUGKS update of
- * Sec. II per block; steps replay a captured CUDA graph.  Each
- * instance's arithmetic is the same as a single solver's Cartesian kernel on the
- * same mesh, so its results do not depend on what else is in the batch.  Instances
+ * Reynolds numbers advanced together; steps replay a captured CUDA graph.  In FP32 a
+ * step is one launch per 96 instances over their (instance, strip, range of rows) items,
+ * one marching warp each.  Instances with a symmetry side or an odd width between
+ * periodic sides, and the 16-bit storages, are stepped by one launch over the (instance,
+ * 16x8 block) work list, one CTA per item (or, if the autotuner prefers it, a fixed grid
+ * of CTAs walking the list).  An instance's arithmetic depends on its own grid only, so
+ * its results do not depend on what else is in the batch.  Instances
  * are admitted while the batch's device pool has room for their state (admission
  * by device-memory footprint) and can be removed at any step boundary, which frees
  * their memory for new ones (continuous batching). */
@@ -328,7 +332,7 @@ typedef struct sdugks_batch_status {
     int64_t pool_bytes;      /* device pool size                                    */
     int64_t pool_used;       /* bytes held by active instances                      */
     int64_t steps;           /* batch steps since creation                          */
-    int32_t grid;            /* CTAs per step launch (the item count if per_item)   */
+    int32_t grid;            /* CTAs per block step launch (the item count if per_item) */
     int32_t ctas_per_sm;     /* resident CTAs per SM of the batched kernel          */
     int32_t graph_steps;     /* steps per captured graph                            */
     int32_t precision;
@@ -372,7 +376,8 @@ int sdugks_batch_get_macros(sdugks_batch *b, int64_t id, double *rho, double *u)
 
 /* Time `steps` steps of each candidate launch form and keep the fastest: one CTA per
  * work item (the default), or a fixed grid of 1, 2 or 4 times the resident CTAs that
- * walks the work list (see sdugks_batch_status.per_item and .grid).  Call with
+ * walks the work list (see sdugks_batch_status.per_item and .grid; instances stepped
+ * by marching warps have one form).  Call with
  * instances admitted.  With one CTA per item, the step graph is captured again after
  * the item count changes (instances admitted or removed). */
 int sdugks_batch_autotune(sdugks_batch *b, int64_t steps);

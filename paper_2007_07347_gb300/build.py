@@ -26,13 +26,14 @@ CU_UNITS = {
     "k_step_fp32.cu": [],
     "k_cart_fp64.cu": ["--fmad=false"],
     "k_cart.cu": [],
+    "k_strip.cu": [],
     "k_util.cu": [],
     "k_residual_noalloc.cu": [],
     "k_batch.cu": [],
     "k_dvm.cu": [],
 }
 CXX_UNITS = ["sdugks_host.cpp"]
-HEADERS = ["sdugks_internal.h", "d2q9.cuh", "step_tiled.cuh", "step_cart.cuh"]
+HEADERS = ["sdugks_internal.h", "d2q9.cuh", "step_tiled.cuh", "step_cart.cuh", "step_strip.cuh"]
 
 
 def _sources():

@@ -1,6 +1,7 @@
 // k_batch.cu -- batched uniform-grid solves: the fused step over an (instance,
-// block) work list, the per-instance residual/mass reduction, and per-instance state
-// set-up and read-out.
+// block) work list (16-bit storages, and FP32 instances that the marching warps of
+// k_strip.cu do not take), the per-instance residual/mass reduction, and per-instance
+// state set-up and read-out.
 #include "step_cart.cuh"
 
 namespace sdugks {

@@ -384,6 +384,8 @@ struct sdugks_solver {
     CartInst ci{};
     int cart_shape = 0;             // Cartesian block shape (CART_TY)
     CartTma *tma = nullptr;         // Cartesian: tensor maps of the TMA staging (nullptr: plain loads)
+    StripInst strip{};              // Cartesian: the solve as the marching form sees it
+    int strip_rows = 0;             // rows per warp of the marching form (0: blocks)
     bool cart_general = false;      // Cartesian: every block on the general code path (one-wave grids)
     double *vol = nullptr, *snap = nullptr, *partial = nullptr, *red = nullptr;
     State st{};
@@ -413,7 +415,9 @@ static cudaError_t launch_one(sdugks_solver *s, cudaStream_t st)
 {
     const int a = s->cur;
     cudaError_t e;
-    if (s->kernel == SDUGKS_KERNEL_CARTESIAN)
+    if (s->strip_rows > 0)
+        e = launch_step_strip(s->strip, s->strip_rows, a, st);
+    else if (s->kernel == SDUGKS_KERNEL_CARTESIAN)
         e = launch_step_cart(s->p.precision, s->cart_shape, s->ci, s->tma, s->cart_general, a, st);
     else if (s->p.precision == P_FP64)
         e = launch_step_tiled_fp64(s->tm, s->coefs, s->st.f[a], s->st.f[1 - a], s->st.W[a], s->st.W[1 - a], st);
@@ -698,6 +702,22 @@ static int create_cart(const sdugks_mesh &m, const CartGrid &g, const sdugks_par
         // MLUPS; 512^2, four waves: 150.1 k against 160.1 k with the interior variant)
         s->cart_general = !use_tma &&
                           s->n_tiles <= (int64_t)n_sm * std::max(1, cart_shape_occupancy(prec, s->cart_shape, false));
+    }
+    // FP32 grids of many waves march (step_strip.cuh) where the two models say that it is
+    // faster: 1.95 us per unit of strip_rows' cost against 54 ps per cell of the blocks'
+    // (16x8, padding included).  GB300, FP32 cavity, blocks / marching in us per step: 384^2
+    // 8.1 / 9.8, 448^2 11.3 / 9.8, 512^2 14.0 / 11.3, 1024^2 48.8 / 34.2, 2048^2 181 / 112.
+    if (!use_tma && !s->cart_general && strip_fits(s->ci, prec)) {
+        const int strips = strip_count(g.nx, g.px);
+        double cost = 0.0;
+        const int rows = strip_rows(strip_slots(), g.ny, [&](int r) { return (int64_t)strips * ((g.ny + r - 1) / r); }, cost);
+        const double blocks = 128.0 * (double)((g.nx + 15) / 16) * (double)((g.ny + 7) / 8);
+        if (rows > 0 && 1.95 * cost < 54e-6 * blocks) s->strip_rows = rows;
+    }
+    if (s->strip_rows > 0) {
+        chk(prepare_strip(), "kernel attributes");
+        if (rc2) { sdugks_solver_destroy(s); return rc2; }
+        fill_strip(s->ci, s->strip);
     }
     // interior blocks staged by tensor copies; the maps hold the fixed addresses of the
     // two state buffers
@@ -1757,6 +1777,7 @@ struct BatchInst {
     size_t off, bytes;
     int64_t admitted_at;            // batch step at admission
     int64_t ntiles;
+    bool strip;                     // steps by marching warps (else by blocks)
     std::vector<int64_t> lattice;   // caller's cell c -> lattice position i + nx j
 };
 
@@ -1785,7 +1806,12 @@ struct sdugks_batch {
     // device tables (fixed addresses, sized for max_inst and max_items)
     CartInst *d_inst = nullptr;
     int2 *d_items = nullptr;
-    int *d_nitems = nullptr;
+    int *d_nitems = nullptr;            // [2]: work items, and those of the instances stepped by blocks (listed first)
+    int2 *d_sitems = nullptr;           // items of the marching warps, by group
+    struct Group { StripGroup g; int64_t first, n; };
+    std::vector<Group> groups;
+    int strip_rows = 0;
+    int64_t n_block = 0;                // items stepped by blocks
     double *d_partial = nullptr, *d_out = nullptr;
     double *h_out = nullptr;            // pinned [max_inst][4]
     double *d_stage = nullptr;          // [max_cells_one][3] staging for add/get
@@ -1795,42 +1821,87 @@ struct sdugks_batch {
     bool per_item = true;                       // one CTA per work item (the grid follows the list)
     int graph_steps = 64;
     cudaGraphExec_t graph = nullptr;
-    int64_t graph_items = -1;                   // the item count the graph's per-item grids were sized for
+    bool graph_strips = false;                  // the graph holds launches of marching warps
+    int64_t n_strip_slots = 1;
 };
 
-// CTAs of a step launch: one per work item (at least one), or the walking form's grid
+// CTAs of a block step launch: one per block item (at least one), or the walking form's grid
 static int batch_launch_grid(const sdugks_batch *b)
 {
-    return b->per_item ? (int)(b->n_items > 0 ? b->n_items : 1) : b->grid;
+    return b->per_item ? (int)(b->n_block > 0 ? b->n_block : 1) : b->grid;
+}
+
+// One step of every instance: the marching warps of each group, then the blocks (the
+// instances are independent; each launch waits for the one before it).
+static cudaError_t batch_launch_step(const sdugks_batch *b, int parity, bool per_item, int grid, cudaStream_t st)
+{
+    cudaError_t e = cudaSuccess;
+    for (const auto &g : b->groups)
+        if (e == cudaSuccess) e = launch_strip_batch(g.g, b->d_sitems + g.first, (int)g.n, b->strip_rows, parity, st);
+    if (e == cudaSuccess && (b->n_block > 0 || b->groups.empty()))
+        e = launch_step_batch(b->prec, b->d_inst, b->d_items, b->d_nitems + 1, grid, per_item, parity, st);
+    return e;
 }
 
 static int batch_upload_tables(sdugks_batch *b)
 {
-    std::vector<CartInst> h;
-    std::vector<int2> items;
-    h.reserve(b->inst.size());
-    for (size_t q = 0; q < b->inst.size(); q++) {
-        CartInst ci = b->inst[q].ci;
-        ci.item0 = (int32_t)items.size();
-        ci.n_items = (int32_t)b->inst[q].ntiles;
-        // item: (instance, block x | block y << 16)
-        const int ntx = (ci.nx + 15) / 16;
-        for (int64_t t = 0; t < b->inst[q].ntiles; t++)
-            items.push_back(make_int2((int)q, (int)(t % ntx) | ((int)(t / ntx) << 16)));
-        b->inst[q].ci.item0 = ci.item0;
-        b->inst[q].ci.n_items = ci.n_items;
-        h.push_back(ci);
+    std::vector<CartInst> h(b->inst.size());
+    std::vector<int2> items, sitems;
+    // instances stepped by blocks first: their items are the head of the list
+    for (const bool strip : {false, true}) {
+        for (size_t q = 0; q < b->inst.size(); q++) {
+            if (b->inst[q].strip != strip) continue;
+            CartInst &ci = b->inst[q].ci;
+            ci.item0 = (int32_t)items.size();
+            ci.n_items = (int32_t)b->inst[q].ntiles;
+            // item: (instance, block x | block y << 16)
+            const int ntx = (ci.nx + 15) / 16;
+            for (int64_t t = 0; t < b->inst[q].ntiles; t++)
+                items.push_back(make_int2((int)q, (int)(t % ntx) | ((int)(t / ntx) << 16)));
+            h[q] = ci;
+        }
+        if (!strip) b->n_block = (int64_t)items.size();
     }
     if ((int64_t)items.size() > b->max_items) return fail(SDUGKS_ERR_FULL, "batch work list full");
     b->n_items = (int64_t)items.size();
-    const int ni = (int)b->n_items;
+    // the marching warps' items, in groups of instances
+    std::vector<const CartInst *> si;
+    int max_ny = 1;
+    for (const auto &i : b->inst)
+        if (i.strip) { si.push_back(&i.ci); max_ny = std::max(max_ny, i.ci.ny); }
+    b->groups.clear();
+    if (!si.empty()) {
+        auto count = [&](int rows) {
+            int64_t n = 0;
+            for (const CartInst *c : si) n += (int64_t)strip_count(c->nx, c->periodic_x != 0) * ((c->ny + rows - 1) / rows);
+            return n > b->max_items ? INT64_MAX / 4096 : n;      // past the list's room
+        };
+        double cost;
+        b->strip_rows = strip_rows(b->n_strip_slots, max_ny, count, cost);
+        for (size_t q = 0; q < si.size(); q++) {
+            if (q % STRIP_GROUP == 0) {
+                b->groups.emplace_back();
+                std::memset(&b->groups.back(), 0, sizeof(b->groups.back()));
+                b->groups.back().first = (int64_t)sitems.size();
+            }
+            auto &G = b->groups.back();
+            const int k = (int)(q % STRIP_GROUP), strips = strip_count(si[q]->nx, si[q]->periodic_x != 0);
+            fill_strip(*si[q], G.g.inst[k]);
+            const int segs = (si[q]->ny + b->strip_rows - 1) / b->strip_rows;
+            for (int t = 0; t < segs; t++)
+                for (int x = 0; x < strips; x++) sitems.push_back(make_int2(k, x | (t << 16)));
+            G.n = (int64_t)sitems.size() - G.first;
+        }
+    }
+    const int ni[2] = {(int)b->n_items, (int)b->n_block};
     if (!h.empty()) CUDA_TRY(cudaMemcpyAsync(b->d_inst, h.data(), h.size() * sizeof(CartInst), cudaMemcpyHostToDevice, b->stream));
     if (!items.empty()) CUDA_TRY(cudaMemcpyAsync(b->d_items, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice, b->stream));
-    CUDA_TRY(cudaMemcpyAsync(b->d_nitems, &ni, sizeof(int), cudaMemcpyHostToDevice, b->stream));
+    if (!sitems.empty()) CUDA_TRY(cudaMemcpyAsync(b->d_sitems, sitems.data(), sitems.size() * sizeof(int2), cudaMemcpyHostToDevice, b->stream));
+    CUDA_TRY(cudaMemcpyAsync(b->d_nitems, ni, sizeof ni, cudaMemcpyHostToDevice, b->stream));
     CUDA_TRY(cudaStreamSynchronize(b->stream));   // the host vectors go out of scope
-    // a graph of per-item launches has grids of the old item count (destroyed after the
-    // synchronisation, so no launch of it is still running)
-    if (b->graph && b->per_item && b->graph_items != b->n_items) {
+    // a graph's launches carry the old list: grids of its item counts, records of its
+    // instances (destroyed after the synchronisation, so no launch of it is still running)
+    if (b->graph && (b->per_item || !b->groups.empty() || b->graph_strips)) {
         cudaGraphExecDestroy(b->graph);
         b->graph = nullptr;
     }
@@ -1859,19 +1930,22 @@ extern "C" int sdugks_batch_create(int64_t pool_bytes, int32_t precision, int32_
     if (e == cudaSuccess) e = cudaMalloc(&b->pool, (size_t)pool_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_inst, sizeof(CartInst) * (size_t)max_instances);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_items, sizeof(int2) * (size_t)b->max_items);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_nitems, sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_sitems, sizeof(int2) * (size_t)(precision == SDUGKS_FP32 ? b->max_items : 1));
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_nitems, 2 * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_partial, sizeof(double) * 4 * (size_t)b->max_items);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_out, sizeof(double) * 4 * (size_t)max_instances);
     if (e == cudaSuccess) e = cudaMallocHost(&b->h_out, sizeof(double) * 4 * (size_t)max_instances);
-    if (e == cudaSuccess) e = cudaMemset(b->d_nitems, 0, sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(b->d_nitems, 0, 2 * sizeof(int));
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = prepare_batch(precision);
+    if (e == cudaSuccess) e = prepare_strip_batch();
     if (e != cudaSuccess)
         return cleanup(fail(e == cudaErrorMemoryAllocation ? SDUGKS_ERR_OOM : SDUGKS_ERR_CUDA, "batch create: %s",
                             cudaGetErrorString(e)));
     b->alloc.reset((size_t)pool_bytes);
     b->ctas_per_sm = batch_ctas_per_sm(precision);
     b->grid = b->n_sm * b->ctas_per_sm;
+    b->n_strip_slots = strip_slots();
     *out = b;
     return SDUGKS_OK;
 }
@@ -1913,6 +1987,7 @@ extern "C" int sdugks_batch_add(sdugks_batch *b, const sdugks_mesh *m, double ta
     bi.admitted_at = b->steps;
     bi.ntiles = (int64_t)((g.nx + 15) / 16) * ((g.ny + BATCH_TY - 1) / BATCH_TY);
     fill_cart_inst(bi.ci, *m, g, tau, dt, pitch, npad);
+    bi.strip = strip_fits(bi.ci, b->prec);
     {
         auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
         const size_t fs = (b->prec == P_BF16DEV || b->prec == P_FP16DEV) ? 2 : 4;
@@ -1983,16 +2058,15 @@ static int batch_ensure_graph(sdugks_batch *b)
     cudaGraph_t g = nullptr;
     CUDA_TRY(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
-    const int grid = batch_launch_grid(b);
     for (int k = 0; k < b->graph_steps && e == cudaSuccess; k++)
-        e = launch_step_batch(b->prec, b->d_inst, b->d_items, b->d_nitems, grid, b->per_item, k & 1, b->cap_stream);
+        e = batch_launch_step(b, k & 1, b->per_item, batch_launch_grid(b), b->cap_stream);
     cudaError_t e2 = cudaStreamEndCapture(b->cap_stream, &g);
     CUDA_TRY(e);
     CUDA_TRY(e2);
     e = cudaGraphInstantiate(&b->graph, g, 0);
     cudaGraphDestroy(g);
     CUDA_TRY(e);
-    b->graph_items = b->n_items;
+    b->graph_strips = !b->groups.empty();
     return SDUGKS_OK;
 }
 
@@ -2004,8 +2078,7 @@ extern "C" int sdugks_batch_step(sdugks_batch *b, int64_t n)
     int64_t left = n;
     if (left >= 2 * b->graph_steps) {
         if (b->cur != 0) {
-            CUDA_TRY(launch_step_batch(b->prec, b->d_inst, b->d_items, b->d_nitems, batch_launch_grid(b),
-                                       b->per_item, b->cur, b->stream));
+            CUDA_TRY(batch_launch_step(b, b->cur, b->per_item, batch_launch_grid(b), b->stream));
             b->cur ^= 1; b->steps++; left--;
         }
         int rc = batch_ensure_graph(b);
@@ -2016,8 +2089,7 @@ extern "C" int sdugks_batch_step(sdugks_batch *b, int64_t n)
         }
     }
     while (left > 0) {
-        CUDA_TRY(launch_step_batch(b->prec, b->d_inst, b->d_items, b->d_nitems, batch_launch_grid(b), b->per_item,
-                                   b->cur, b->stream));
+        CUDA_TRY(batch_launch_step(b, b->cur, b->per_item, batch_launch_grid(b), b->stream));
         b->cur ^= 1; b->steps++; left--;
     }
     return SDUGKS_OK;
@@ -2078,7 +2150,7 @@ extern "C" int sdugks_batch_autotune(sdugks_batch *b, int64_t steps)
     // candidates: one CTA per item (mult 0), then the walking form at 1, 2 and 4 times
     // the resident CTAs
     const int base = b->n_sm * b->ctas_per_sm;
-    const int item_grid = (int)(b->n_items > 0 ? b->n_items : 1);
+    const int item_grid = (int)(b->n_block > 0 ? b->n_block : 1);
     int best = 0;
     float best_ms = 1e30f;
     for (int mult : {0, 1, 2, 4}) {
@@ -2086,10 +2158,10 @@ extern "C" int sdugks_batch_autotune(sdugks_batch *b, int64_t steps)
         const int grid = per_item ? item_grid : base * mult;
         // steps in pairs so that the buffer parity is unchanged
         for (int64_t k = 0; k < 2; k++)
-            launch_step_batch(b->prec, b->d_inst, b->d_items, b->d_nitems, grid, per_item, (b->cur + k) & 1, b->stream);
+            batch_launch_step(b, (b->cur + k) & 1, per_item, grid, b->stream);
         cudaEventRecord(e0, b->stream);
         for (int64_t k = 0; k < 2 * steps; k++)
-            launch_step_batch(b->prec, b->d_inst, b->d_items, b->d_nitems, grid, per_item, (b->cur + k) & 1, b->stream);
+            batch_launch_step(b, (b->cur + k) & 1, per_item, grid, b->stream);
         cudaEventRecord(e1, b->stream);
         cudaError_t e = cudaEventSynchronize(e1);
         float ms = 0;
@@ -2120,7 +2192,7 @@ extern "C" int sdugks_batch_info(const sdugks_batch *b, sdugks_batch_status *o)
     o->pool_bytes = (int64_t)b->alloc.cap();
     o->pool_used = (int64_t)b->alloc.used();
     o->steps = b->steps;
-    o->grid = batch_launch_grid(b);
+    o->grid = b->per_item ? (int)std::max<int64_t>(b->n_items, 1) : b->grid;
     o->ctas_per_sm = b->ctas_per_sm;
     o->graph_steps = b->graph_steps;
     o->precision = b->prec;
@@ -2138,6 +2210,7 @@ extern "C" void sdugks_batch_destroy(sdugks_batch *b)
     cudaFree(b->pool);
     cudaFree(b->d_inst);
     cudaFree(b->d_items);
+    cudaFree(b->d_sitems);
     cudaFree(b->d_nitems);
     cudaFree(b->d_partial);
     cudaFree(b->d_out);

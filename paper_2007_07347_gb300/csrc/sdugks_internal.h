@@ -144,6 +144,54 @@ cudaError_t make_cart_tma(int prec, int shape, const CartInst &m, CartTma &out);
 cudaError_t launch_step_cart(int prec, int shape, const CartInst &m, const CartTma *tma, bool general, int parity,
                              cudaStream_t st);
 int cart_shape_occupancy(int prec, int shape, bool tma);   // resident CTAs per SM
+// One uniform-grid solve as the marching form sees it (FP32 storage; no symmetry side,
+// an even nx where x is periodic): the grid and its side rules, the ping-pong state, and
+// the step's constants, each twice (one operand of a paired instruction).
+struct StripInst {
+    int32_t nx, ny, pitch, npad, periodic_x, periodic_y;
+    int32_t side_kind[4];
+    float side_par[4][3], side_drho[4];
+    float sb, sc, len_dtV[2];                  // b, c; lengths of faces of constant x, y times dt / V
+    float *f[2];
+    double *W[2];
+    float2 a, b, inv, ri;                      // inv = 1 / (1 + r), ri = r inv
+    float2 g[2], bg[2];                        // faces of constant x, y: c len dt/V, b c len dt/V
+    float2 xdt[2], xh[2], xo[2];               // dt, h/2, h/2 - dt along x, times 1/(2 dx); [1] negated
+    float2 ydt[2], yh[2], yo[2];
+};
+bool strip_fits(const CartInst &m, int prec);                // the marching form takes this solve
+void fill_strip(const CartInst &m, StripInst &s);
+int strip_count(int nx, bool periodic_x);                    // 60-column strips of a grid
+// rows per warp for a set of grids (strips x rows, as counted by `items(rows)`) that fill
+// `slots` resident warps best, and the model's time of a step in row units
+template <class Items> inline int strip_rows(int64_t slots, int max_ny, Items &&items, double &cost)
+{
+    // A range of rows costs rows + 2 units (two rows' worth for its halo and its start).
+    // A step is half whole waves, half work that fills the slots evenly: with items / slots
+    // = r, (rows + 2) (ceil(r) + max(1, r)) / 2.  Fits 40 measured (size, rows) pairs from
+    // 448^2 to 2048^2 within 6 % at 1.8 to 2.1 us a unit (GB300).
+    int best = 0;
+    cost = 1e300;
+    for (int rows = 1; rows <= max_ny && rows <= 256; rows += 1 + rows / 16) {
+        if ((max_ny + rows - 1) / rows > 32767) continue;
+        const double r = (double)items(rows) / (double)slots;
+        const double c = (rows + 2) * 0.5 * ((double)(int64_t)(r + 0.999999) + (r > 1.0 ? r : 1.0));
+        if (c < cost) { cost = c; best = rows; }
+    }
+    return best;                               // 0: no range fits
+}
+cudaError_t prepare_strip();
+cudaError_t launch_step_strip(const StripInst &s, int rows, int parity, cudaStream_t st);
+int strip_slots();                                           // resident warps of the device
+// batched: a group of instances, handed to the kernel by value (constant memory), and its
+// (instance of the group, strip | range << 16) items in device memory, one warp each
+constexpr int STRIP_GROUP = 96;
+struct StripGroup {
+    StripInst inst[STRIP_GROUP];
+};
+static_assert(sizeof(StripGroup) <= 32000, "a group is a kernel parameter");
+cudaError_t prepare_strip_batch();
+cudaError_t launch_strip_batch(const StripGroup &g, const int2 *items, int n_items, int rows, int parity, cudaStream_t st);
 // batched: every (instance, tile) item of the list, one per CTA (per_item: grid >= the
 // item count) or grid-stride over a fixed grid
 cudaError_t prepare_batch(int prec);
