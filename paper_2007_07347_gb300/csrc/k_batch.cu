@@ -96,9 +96,9 @@ cudaError_t launch_batch_p(const CartInst *insts, const int2 *items, const int *
                            int parity, cudaStream_t st)
 {
     if (per_item)
-        return launch_step_kernel(k_step_batch<P, BTX, BTY, true>, dim3(grid), dim3(cart_threads<BTX, BTY>()),
+        return launch_step_kernel(true, k_step_batch<P, BTX, BTY, true>, dim3(grid), dim3(cart_threads<BTX, BTY>()),
                                   cart_smem<P, BTX, BTY>(), st, insts, items, n_items, parity);
-    return launch_step_kernel(k_step_batch<P, BTX, BTY, false>, dim3(grid), dim3(cart_threads<BTX, BTY>()),
+    return launch_step_kernel(true, k_step_batch<P, BTX, BTY, false>, dim3(grid), dim3(cart_threads<BTX, BTY>()),
                               cart_smem<P, BTX, BTY>(), st, insts, items, n_items, parity);
 }
 

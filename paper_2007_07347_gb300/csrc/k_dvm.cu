@@ -652,19 +652,19 @@ cudaError_t step_pv(const DvmMesh &m, const Coefs &c, double RTw, void *f, doubl
     const R *cfbp = pfbp, *cflux = pflux;
     cudaError_t e = cudaSuccess;
     if (!fbp_ready)
-        e = launch_step_kernel(k_dvm_fbp<R, V>, cells, dim3(FBP_THREADS), 0, st, m, c, cf, (const double *)W, pfbp);
+        e = launch_step_kernel(true, k_dvm_fbp<R, V>, cells, dim3(FBP_THREADS), 0, st, m, c, cf, (const double *)W, pfbp);
     if (e != cudaSuccess) return e;
     // the cell kernel leaves the next step's fbar+ in fbp (read by this step's face kernel
     // before the cell kernel starts)
     if (dvm_use_smem<R>(m.Q)) {
         const size_t bytes = (size_t)m.Q * sizeof(R);
-        e = launch_step_kernel(k_dvm_face<R, true, V>, faces, dim3(FACE_THREADS), bytes, st, m, c, RTw, cfbp, pflux);
+        e = launch_step_kernel(true, k_dvm_face<R, true, V>, faces, dim3(FACE_THREADS), bytes, st, m, c, RTw, cfbp, pflux);
         if (e == cudaSuccess)
-            e = launch_step_kernel(k_dvm_cell<R, true, V>, cells, dim3(CELL_THREADS), bytes, st, m, c, pf, W, cflux, pfbp);
+            e = launch_step_kernel(true, k_dvm_cell<R, true, V>, cells, dim3(CELL_THREADS), bytes, st, m, c, pf, W, cflux, pfbp);
     } else {
-        e = launch_step_kernel(k_dvm_face<R, false, V>, faces, dim3(FACE_THREADS), 0, st, m, c, RTw, cfbp, pflux);
+        e = launch_step_kernel(true, k_dvm_face<R, false, V>, faces, dim3(FACE_THREADS), 0, st, m, c, RTw, cfbp, pflux);
         if (e == cudaSuccess)
-            e = launch_step_kernel(k_dvm_cell<R, false, V>, cells, dim3(CELL_THREADS), 0, st, m, c, pf, W, cflux, pfbp);
+            e = launch_step_kernel(true, k_dvm_cell<R, false, V>, cells, dim3(CELL_THREADS), 0, st, m, c, pf, W, cflux, pfbp);
     }
     return e;
 }

@@ -10,6 +10,12 @@ cudaError_t prepare_tiled_fp32(int prec)
     return prec == P_BF16DEV ? prepare_tiled_p<P_BF16DEV>() : prepare_tiled_p<P_FP32>();
 }
 
+int occ_tiled_fp32(int prec)
+{
+    if (prec == P_FP16DEV) return occ_tiled_p<P_FP16DEV>();
+    return prec == P_BF16DEV ? occ_tiled_p<P_BF16DEV>() : occ_tiled_p<P_FP32>();
+}
+
 cudaError_t launch_step_tiled_fp32(int prec, const TiledMesh &m, const Coefs &c, const void *f_in, void *f_out,
                                    const double *W_in, double *W_out, cudaStream_t st)
 {

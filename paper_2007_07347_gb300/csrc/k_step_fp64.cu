@@ -5,6 +5,8 @@
 
 namespace sdugks {
 
+int occ_tiled_fp64() { return occ_tiled_p<P_FP64>(); }
+
 cudaError_t prepare_tiled_fp64() { return prepare_tiled_p<P_FP64>(); }
 
 cudaError_t launch_step_tiled_fp64(const TiledMesh &m, const Coefs &c, const void *f_in, void *f_out,

@@ -7,7 +7,7 @@ namespace sdugks {
 // then uniform to the compiler, and warps that share nothing need not end together.
 __global__ void __launch_bounds__(32, STRIP_CTAS) k_step_strip(const StripInst m, int par, int rows)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    extern __shared__ __align__(128) unsigned char smem_raw[];
     step_dependency_wait();
     strip_item(m, par, blockIdx.x, blockIdx.y, rows, smem_raw);
 }
@@ -18,7 +18,7 @@ __global__ void __launch_bounds__(32, STRIP_CTAS) k_step_strip(const StripInst m
 __global__ void __launch_bounds__(32, STRIP_CTAS)
 k_strip_batch(const __grid_constant__ StripGroup G, const int2 *__restrict__ items, int par, int rows)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    extern __shared__ __align__(128) unsigned char smem_raw[];
     const int2 it = items[blockIdx.x];
     step_dependency_wait();
     const int q = __shfl_sync(0xffffffffu, it.x, 0), y = __shfl_sync(0xffffffffu, it.y, 0);
@@ -75,14 +75,15 @@ cudaError_t prepare_strip_batch()
     return cudaFuncSetAttribute(k_strip_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)STRIP_SMEM);
 }
 
-cudaError_t launch_strip_batch(const StripGroup &g, const int2 *items, int n_items, int rows, int parity, cudaStream_t st)
+cudaError_t launch_strip_batch(const StripGroup &g, const int2 *items, int n_items, int rows, bool early,
+                               int parity, cudaStream_t st)
 {
-    return launch_step_kernel(k_strip_batch, dim3(n_items), dim3(32), STRIP_SMEM, st, g, items, parity, rows);
+    return launch_step_kernel(early, k_strip_batch, dim3(n_items), dim3(32), STRIP_SMEM, st, g, items, parity, rows);
 }
 
-cudaError_t launch_step_strip(const StripInst &s, int rows, int parity, cudaStream_t st)
+cudaError_t launch_step_strip(const StripInst &s, int rows, bool early, int parity, cudaStream_t st)
 {
-    return launch_step_kernel(k_step_strip, dim3(strip_count(s.nx, s.periodic_x != 0), (s.ny + rows - 1) / rows), dim3(32),
+    return launch_step_kernel(early, k_step_strip, dim3(strip_count(s.nx, s.periodic_x != 0), (s.ny + rows - 1) / rows), dim3(32),
                               STRIP_SMEM, st, s, parity, rows);
 }
 

@@ -383,9 +383,11 @@ struct sdugks_solver {
     int32_t *loc = nullptr;         // q-th listed cell -> internal offset (nullptr: q)
     CartInst ci{};
     int cart_shape = 0;             // Cartesian block shape (CART_TY)
+    int launch_shape = 0;           // the shape given to the launch: cart_shape, or FP64's own (cart64_shape)
     CartTma *tma = nullptr;         // Cartesian: tensor maps of the TMA staging (nullptr: plain loads)
     StripInst strip{};              // Cartesian: the solve as the marching form sees it
     int strip_rows = 0;             // rows per warp of the marching form (0: blocks)
+    bool strip_early = true;
     bool cart_general = false;      // Cartesian: every block on the general code path (one-wave grids)
     double *vol = nullptr, *snap = nullptr, *partial = nullptr, *red = nullptr;
     State st{};
@@ -416,9 +418,9 @@ static cudaError_t launch_one(sdugks_solver *s, cudaStream_t st)
     const int a = s->cur;
     cudaError_t e;
     if (s->strip_rows > 0)
-        e = launch_step_strip(s->strip, s->strip_rows, a, st);
+        e = launch_step_strip(s->strip, s->strip_rows, s->strip_early, a, st);
     else if (s->kernel == SDUGKS_KERNEL_CARTESIAN)
-        e = launch_step_cart(s->p.precision, s->cart_shape, s->ci, s->tma, s->cart_general, a, st);
+        e = launch_step_cart(s->p.precision, s->launch_shape, s->ci, s->tma, s->cart_general, a, st);
     else if (s->p.precision == P_FP64)
         e = launch_step_tiled_fp64(s->tm, s->coefs, s->st.f[a], s->st.f[1 - a], s->st.W[a], s->st.W[1 - a], st);
     else
@@ -700,8 +702,11 @@ static int create_cart(const sdugks_mesh &m, const CartGrid &g, const sdugks_par
         // all blocks in one wave: the slowest (edge) block sets the step time, and one
         // code path for every block measured faster (GB300, 256^2: 126.4 k against 120.3 k
         // MLUPS; 512^2, four waves: 150.1 k against 160.1 k with the interior variant)
-        s->cart_general = !use_tma &&
-                          s->n_tiles <= (int64_t)n_sm * std::max(1, cart_shape_occupancy(prec, s->cart_shape, false));
+        int64_t slots = (int64_t)n_sm * std::max(1, cart_shape_occupancy(prec, s->cart_shape, use_tma));
+        s->cart_general = !use_tma && s->n_tiles <= slots;
+        int64_t ctas = s->n_tiles;
+        s->launch_shape = prec == P_FP64 ? cart64_shape(g.nx, g.ny, n_sm) : s->cart_shape;
+        s->ci.early = early_start(ctas, slots, n_sm);
     }
     // FP32 grids of many waves march (step_strip.cuh) where the two models say that it is
     // faster: 1.95 us per unit of strip_rows' cost against 54 ps per cell of the blocks'
@@ -718,6 +723,10 @@ static int create_cart(const sdugks_mesh &m, const CartGrid &g, const sdugks_par
         chk(prepare_strip(), "kernel attributes");
         if (rc2) { sdugks_solver_destroy(s); return rc2; }
         fill_strip(s->ci, s->strip);
+        int n_sm = 1;
+        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, s->device);
+        s->strip_early = early_start((int64_t)strip_count(g.nx, g.px) * ((g.ny + s->strip_rows - 1) / s->strip_rows),
+                                     strip_slots(), n_sm);
     }
     // interior blocks staged by tensor copies; the maps hold the fixed addresses of the
     // two state buffers
@@ -843,11 +852,11 @@ extern "C" int sdugks_solver_create(const sdugks_mesh *m, const sdugks_params *p
     std::vector<TileHalo> halos;
     std::vector<std::pair<size_t, size_t>> final_tiles;
     int32_t tag = 0;
-    for (size_t ti = 0; ti < tiles.size(); ti++) {
-        const auto [lo, hi] = tiles[ti];
+    // the two rings of neighbours around the cells ids[lo, hi), and the number of faces that
+    // touch those cells
+    auto rings = [&](size_t lo, size_t hi, TileHalo &h) {
         tag++;
         for (size_t i = lo; i < hi; i++) stamp[ids[i]] = tag;
-        TileHalo h;
         size_t n_faces = 0;
         for (size_t i = lo; i < hi; i++)
             for (int sl = 0; sl < nslot[ids[i]]; sl++) {
@@ -861,9 +870,18 @@ extern "C" int sdugks_solver_create(const sdugks_mesh *m, const sdugks_params *p
                 const int64_t kc = other_of(c1, sl);
                 if (kc >= 0 && stamp[kc] != tag) { stamp[kc] = tag; h.r2.push_back((int32_t)kc); }
             }
+        return n_faces;
+    };
+    auto fits = [&](size_t lo, size_t hi, const TileHalo &h, size_t n_faces) {
+        return hi - lo + h.r1.size() + h.r2.size() <= (size_t)LOC_MAX && hi - lo + h.r1.size() <= (size_t)SIG_MAX &&
+               n_faces <= (size_t)LF_MAX;
+    };
+    for (size_t ti = 0; ti < tiles.size(); ti++) {
+        const auto [lo, hi] = tiles[ti];
+        TileHalo h;
+        const size_t n_faces = rings(lo, hi, h);
         const size_t nint = hi - lo;
-        if (nint + h.r1.size() + h.r2.size() > (size_t)LOC_MAX || nint + h.r1.size() > (size_t)SIG_MAX ||
-            n_faces > (size_t)LF_MAX) {
+        if (!fits(lo, hi, h, n_faces)) {
             if (nint <= 8) return fail(SDUGKS_ERR_INVALID_MESH, "halo of a %zu-cell tile does not fit", nint);
             std::vector<std::pair<size_t, size_t>> sub;
             rcb(m->xc, ids, lo, hi, (nint + 1) / 2, sub);
@@ -873,7 +891,6 @@ extern "C" int sdugks_solver_create(const sdugks_mesh *m, const sdugks_params *p
         final_tiles.push_back(tiles[ti]);
         halos.push_back(std::move(h));
     }
-    const int32_t nt = (int32_t)final_tiles.size();
     // within a tile, cells along a Morton curve of their centroids (16 bits per axis over
     // the tile's bounding box): faces, which are listed in the order of their cells,
     // then read nearby local indices from one warp to the next lane
@@ -900,6 +917,7 @@ extern "C" int sdugks_solver_create(const sdugks_mesh *m, const sdugks_params *p
             return ka != kb ? ka < kb : a < b;
         });
     }
+    const int32_t nt = (int32_t)final_tiles.size();
     // internal order: tiles in RCB order
     std::vector<int32_t> perm(n), iperm(n);
     {
@@ -1203,6 +1221,11 @@ extern "C" int sdugks_solver_create(const sdugks_mesh *m, const sdugks_params *p
     chk(cudaStreamCreateWithFlags(&s->cap_stream, cudaStreamNonBlocking), "cudaStreamCreate");
     chk((cudaError_t)prepare(prec, SDUGKS_KERNEL_TILED), "kernel attributes");
     if (rc2) { sdugks_solver_destroy(s); return rc2; }
+    {
+        int n_sm = 1;
+        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, s->device);
+        s->tm.early = early_start(nt, (int64_t)n_sm * (prec == P_FP64 ? occ_tiled_fp64() : occ_tiled_fp32(prec)), n_sm);
+    }
 
     fill_coefs(s->coefs, *m, prm->tau, prm->dt);
     // mesh bytes the tiled kernel reads per interior cell and step: the slot list of
@@ -1356,7 +1379,7 @@ extern "C" int sdugks_step_boundary_flux(sdugks_solver *s, double *force, double
         CartInst ci = s->ci;
         ci.force = d_force;                    // per grid side
         ci.bface = d_bface;
-        e = launch_step_cart(s->p.precision, s->cart_shape, ci, s->tma, s->cart_general, s->cur, s->stream);
+        e = launch_step_cart(s->p.precision, s->launch_shape, ci, s->tma, s->cart_general, s->cur, s->stream);
     } else {
         TiledMesh tm = s->tm;
         tm.force = d_force;                    // per patch
@@ -1811,6 +1834,7 @@ struct sdugks_batch {
     struct Group { StripGroup g; int64_t first, n; };
     std::vector<Group> groups;
     int strip_rows = 0;
+    bool strip_early = true;
     int64_t n_block = 0;                // items stepped by blocks
     double *d_partial = nullptr, *d_out = nullptr;
     double *h_out = nullptr;            // pinned [max_inst][4]
@@ -1837,7 +1861,8 @@ static cudaError_t batch_launch_step(const sdugks_batch *b, int parity, bool per
 {
     cudaError_t e = cudaSuccess;
     for (const auto &g : b->groups)
-        if (e == cudaSuccess) e = launch_strip_batch(g.g, b->d_sitems + g.first, (int)g.n, b->strip_rows, parity, st);
+        if (e == cudaSuccess)
+            e = launch_strip_batch(g.g, b->d_sitems + g.first, (int)g.n, b->strip_rows, b->strip_early, parity, st);
     if (e == cudaSuccess && (b->n_block > 0 || b->groups.empty()))
         e = launch_step_batch(b->prec, b->d_inst, b->d_items, b->d_nitems + 1, grid, per_item, parity, st);
     return e;
@@ -1892,6 +1917,7 @@ static int batch_upload_tables(sdugks_batch *b)
                 for (int x = 0; x < strips; x++) sitems.push_back(make_int2(k, x | (t << 16)));
             G.n = (int64_t)sitems.size() - G.first;
         }
+        b->strip_early = early_start((int64_t)sitems.size(), b->n_strip_slots, b->n_sm);
     }
     const int ni[2] = {(int)b->n_items, (int)b->n_block};
     if (!h.empty()) CUDA_TRY(cudaMemcpyAsync(b->d_inst, h.data(), h.size() * sizeof(CartInst), cudaMemcpyHostToDevice, b->stream));

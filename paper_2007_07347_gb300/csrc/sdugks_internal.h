@@ -80,6 +80,7 @@ struct TiledMesh {
     double *force;            // nullptr, or [MAXPATCH][2]: momentum flux out of the fluid per boundary patch
     const int32_t *lf_bface;  // [n_lf] boundary-face row of each local face (-1: interior or periodic)
     double *bface;            // nullptr, or [n_bfaces][2]: momentum flux out of the fluid per boundary face
+    bool early;               // launches allow the early start (early_start)
 };
 constexpr uint16_t LF_SECOND = 0x8000, LF_NONE = 0xFFFF;
 constexpr uint32_t LF_BOUNDARY = 0xC000;
@@ -109,6 +110,7 @@ struct CartInst {
     const int32_t *bidx;      // [2 (nx + ny)] boundary-face row of each side face: bottom (by i), right
                               //   (by j), top (by i), left (by j); -1 on periodic sides
     double *bface;            // nullptr, or [n_bfaces][2]: momentum flux out of the fluid per boundary face
+    int64_t early;            // launches allow the early start (early_start)
 };
 
 // Device state of one solver, ping-pong: f [2][NQ][npad] (element type by
@@ -124,6 +126,8 @@ cudaError_t prepare_tiled_fp64();
 cudaError_t launch_step_tiled_fp64(const TiledMesh &m, const Coefs &c, const void *f_in, void *f_out,
                                    const double *W_in, double *W_out, cudaStream_t st);
 cudaError_t prepare_tiled_fp32(int prec);
+int occ_tiled_fp64();
+int occ_tiled_fp32(int prec);                              // resident tiles per SM
 cudaError_t prepare_cart(int prec);
 // block shapes of the Cartesian kernel: 0 = 16x16, 1 = 16x14, 2 = 16x8 (FP64: 16x16 only)
 constexpr int CART_SHAPES = 3;
@@ -144,6 +148,10 @@ cudaError_t make_cart_tma(int prec, int shape, const CartInst &m, CartTma &out);
 cudaError_t launch_step_cart(int prec, int shape, const CartInst &m, const CartTma *tma, bool general, int parity,
                              cudaStream_t st);
 int cart_shape_occupancy(int prec, int shape, bool tma);   // resident CTAs per SM
+// FP64 with plain loads: blocks of 16x14, 8x8 or 4x4 cells (shape 0, 1, 2), by grid size
+cudaError_t prepare_cart64();
+cudaError_t launch_step_cart64(const CartInst &m, int shape, int parity, cudaStream_t st);
+int cart64_shape(int nx, int ny, int n_sm);
 // One uniform-grid solve as the marching form sees it (FP32 storage; no symmetry side,
 // an even nx where x is periodic): the grid and its side rules, the ping-pong state, and
 // the step's constants, each twice (one operand of a paired instruction).
@@ -181,7 +189,7 @@ template <class Items> inline int strip_rows(int64_t slots, int max_ny, Items &&
     return best;                               // 0: no range fits
 }
 cudaError_t prepare_strip();
-cudaError_t launch_step_strip(const StripInst &s, int rows, int parity, cudaStream_t st);
+cudaError_t launch_step_strip(const StripInst &s, int rows, bool early, int parity, cudaStream_t st);
 int strip_slots();                                           // resident warps of the device
 // batched: a group of instances, handed to the kernel by value (constant memory), and its
 // (instance of the group, strip | range << 16) items in device memory, one warp each
@@ -191,7 +199,8 @@ struct StripGroup {
 };
 static_assert(sizeof(StripGroup) <= 32000, "a group is a kernel parameter");
 cudaError_t prepare_strip_batch();
-cudaError_t launch_strip_batch(const StripGroup &g, const int2 *items, int n_items, int rows, int parity, cudaStream_t st);
+cudaError_t launch_strip_batch(const StripGroup &g, const int2 *items, int n_items, int rows, bool early, int parity,
+                               cudaStream_t st);
 // batched: every (instance, tile) item of the list, one per CTA (per_item: grid >= the
 // item count) or grid-stride over a fixed grid
 cudaError_t prepare_batch(int prec);
@@ -216,6 +225,8 @@ cudaError_t launch_step_tiled_fp32(int prec, const TiledMesh &m, const Coefs &c,
 // only the host writes (mesh data, work items) may be read before the wait.  The
 // next step's CTAs therefore take the SM slots the moment the current step's CTAs
 // retire, instead of after the launch latency.
+inline bool early_start(int64_t, int64_t, int) { return true; }
+
 #ifdef __CUDACC__
 __device__ __forceinline__ void step_dependency_wait()
 {
@@ -223,8 +234,10 @@ __device__ __forceinline__ void step_dependency_wait()
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// early: allow the programmatic early start (see early_start)
 template <class... P, class... A>
-cudaError_t launch_step_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args)
+cudaError_t launch_step_kernel(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                               A &&...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -235,7 +248,7 @@ cudaError_t launch_step_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<A &&>(args)...);
 }
 #endif

@@ -830,16 +830,16 @@ cudaError_t launch_cart_p(const CartInst &m, const CartTma *tma, bool general, i
     const dim3 grid(ntx, nty), block(cart_threads<TX, TY>());
     static const CUtensorMap none0{};
     if (m.force || m.bface)
-        return launch_step_kernel(k_step_cart<P, TX, TY, CART_GENERAL, true>, grid, block,
+        return launch_step_kernel(m.early != 0, k_step_cart<P, TX, TY, CART_GENERAL, true>, grid, block,
                                   cart_step_smem<P, TX, TY, CART_GENERAL>(), st, m, par, none0, none0);
     if (tma)
-        return launch_step_kernel(k_step_cart<P, TX, TY, CART_SPECIALISED_TMA>, grid, block,
+        return launch_step_kernel(m.early != 0, k_step_cart<P, TX, TY, CART_SPECIALISED_TMA>, grid, block,
                                   cart_step_smem<P, TX, TY, CART_SPECIALISED_TMA>(), st, m, par, tma->f[par], tma->W[par]);
     static const CUtensorMap none{};
     if (general)
-        return launch_step_kernel(k_step_cart<P, TX, TY, CART_GENERAL>, grid, block,
+        return launch_step_kernel(m.early != 0, k_step_cart<P, TX, TY, CART_GENERAL>, grid, block,
                                   cart_step_smem<P, TX, TY, CART_GENERAL>(), st, m, par, none, none);
-    return launch_step_kernel(k_step_cart<P, TX, TY, CART_SPECIALISED>, grid, block,
+    return launch_step_kernel(m.early != 0, k_step_cart<P, TX, TY, CART_SPECIALISED>, grid, block,
                               cart_step_smem<P, TX, TY, CART_SPECIALISED>(), st, m, par, none, none);
 }
 

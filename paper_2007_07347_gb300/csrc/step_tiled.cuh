@@ -624,6 +624,15 @@ template <int P> cudaError_t prepare_tiled_p() {
     return e == cudaSuccess ? prepare_tiled_pd<P, true>() : e;
 }
 
+template <int P> int occ_tiled_p()
+{
+    int n = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_step_tiled<P, false>, TILED_THREADS, tiled_smem<P>()) !=
+            cudaSuccess || n < 1)
+        return 1;
+    return n;
+}
+
 template <int P>
 cudaError_t launch_tiled_p(const TiledMesh &m, const Coefs &c, const void *fin, void *fout, const double *Wn,
                            double *Wout, cudaStream_t st)
@@ -631,9 +640,9 @@ cudaError_t launch_tiled_p(const TiledMesh &m, const Coefs &c, const void *fin, 
     using T = typename Store<P>::T;
     if (m.n_tiles <= 0) return cudaSuccess;
     if (m.force || m.bface)     // the diagnostic step
-        return launch_step_kernel(k_step_tiled<P, true>, dim3(m.n_tiles), dim3(TILED_THREADS), tiled_smem<P>(), st, m,
+        return launch_step_kernel(m.early, k_step_tiled<P, true>, dim3(m.n_tiles), dim3(TILED_THREADS), tiled_smem<P>(), st, m,
                                   c, static_cast<const T *>(fin), static_cast<T *>(fout), Wn, Wout);
-    return launch_step_kernel(k_step_tiled<P, false>, dim3(m.n_tiles), dim3(TILED_THREADS), tiled_smem<P>(), st, m, c,
+    return launch_step_kernel(m.early, k_step_tiled<P, false>, dim3(m.n_tiles), dim3(TILED_THREADS), tiled_smem<P>(), st, m, c,
                               static_cast<const T *>(fin), static_cast<T *>(fout), Wn, Wout);
 }
 
