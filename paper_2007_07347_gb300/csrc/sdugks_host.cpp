@@ -706,6 +706,27 @@ static int create_cart(const sdugks_mesh &m, const CartGrid &g, const sdugks_par
         s->cart_general = !use_tma && s->n_tiles <= slots;
         int64_t ctas = s->n_tiles;
         s->launch_shape = prec == P_FP64 ? cart64_shape(g.nx, g.ny, n_sm) : s->cart_shape;
+        if (prec == P_FP32 && !use_tma && prm->tile_cells == 0) {
+            // FP32 with plain loads: the time of one step (us, GB300, up to two waves) is
+            // 2.7 plus a shape's time per block of the fullest SM, for the waves that it
+            // takes.  Measured, 16x14 / 16x8 blocks: 64^2 3.5 / 3.1, 128^2 3.6 / 3.1, 192^2
+            // 4.4 / 3.5, 224^2 4.6 / 4.0, 256^2 4.46 / 4.76, 320^2 7.3 / 6.6, 384^2 9.4 / 8.1.
+            // (cart_shape, the model for all shapes of any size, stays what info and a raw
+            // state's header name.)
+            const double per_block[CART_SHAPES] = {1.02, 0.87, 0.48};
+            double best = 1e300;
+            for (int sh = 0; sh < CART_SHAPES; sh++) {
+                const int64_t occ = std::max(1, cart_shape_occupancy(prec, sh, false));
+                const int64_t tiles = (int64_t)((g.nx + 15) / 16) * ((g.ny + CART_TY[sh] - 1) / CART_TY[sh]);
+                const double r = (double)tiles / (double)(occ * n_sm);
+                const double k = (double)std::min<int64_t>(occ, (tiles + n_sm - 1) / n_sm);
+                const double cost = (2.7 + k * per_block[sh]) * 0.5 * (std::max(1.0, r) + std::ceil(r));
+                if (cost < best) {
+                    best = cost; s->launch_shape = sh;
+                    ctas = tiles; slots = occ * n_sm;
+                }
+            }
+        }
         s->ci.early = early_start(ctas, slots, n_sm);
     }
     // FP32 grids of many waves march (step_strip.cuh) where the two models say that it is
