@@ -89,7 +89,9 @@ typedef struct sdugks_params {
     int32_t kernel;      /* SDUGKS_KERNEL_*                                        */
     int32_t tile_cells;  /* tiled kernel: cells per tile (16..128); Cartesian kernel (FP32,
                             bf16 and fp16 storage): 256, 224 or 128 for 16x16, 16x14 or 16x8 blocks;
-                            0 = chosen from the grid size (Cartesian) or 128 (tiled).  With
+                            0 = chosen from the grid size (Cartesian) or 128 (tiled; meshes
+                            that fill less than half the device run on half tiles, in the
+                            same cell order).  With
                             plain loads, FP32 grids of many waves of blocks (about 430^2
                             cells and up, no symmetry side) are stepped by marching warps
                             instead; the blocks then run the diagnostic steps only */

@@ -938,6 +938,33 @@ extern "C" int sdugks_solver_create(const sdugks_mesh *m, const sdugks_params *p
             return ka != kb ? ka < kb : a < b;
         });
     }
+    // Small meshes, tile size left open: where twice the tiles still fit the device at once, the
+    // step runs on half tiles (halves of the Morton curve, so the cell order, and with it a
+    // raw state, stays that of the whole tiles).  More SMs then share the work, and the
+    // SMs that hold two tiles hold less.  GB300, FP32 O-meshes, us per step with tiles of
+    // 128 / of 64 cells: 128x64 5.5 / 4.5, 208x104 6.1 / 5.6, 256x128 6.2 / 5.5; past one wave the
+    // larger halos lose: 304x152 7.6 / 8.1, 512x256 13.2 / 16.4.
+    if (prm->tile_cells == 0) {
+        int dev = 0, n_sm = 0;
+        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+        if (n_sm > 0 && prepare(prm->precision, SDUGKS_KERNEL_TILED) == 0) {
+            const int64_t slots = (int64_t)n_sm * (prm->precision == P_FP64 ? occ_tiled_fp64() : occ_tiled_fp32(prm->precision));
+            std::vector<std::pair<size_t, size_t>> half;
+            std::vector<TileHalo> hh;
+            bool ok = 2 * (int64_t)final_tiles.size() <= slots;
+            for (size_t ti = 0; ok && ti < final_tiles.size(); ti++) {
+                const size_t lo = final_tiles[ti].first, hi = final_tiles[ti].second, mid = lo + (hi - lo + 1) / 2;
+                for (const auto &q : {std::make_pair(lo, mid), std::make_pair(mid, hi)}) {
+                    if (q.first == q.second) continue;
+                    TileHalo h;
+                    ok = ok && fits(q.first, q.second, h, rings(q.first, q.second, h));
+                    half.push_back(q);
+                    hh.push_back(std::move(h));
+                }
+            }
+            if (ok) { final_tiles = std::move(half); halos = std::move(hh); }
+        }
+    }
     const int32_t nt = (int32_t)final_tiles.size();
     // internal order: tiles in RCB order
     std::vector<int32_t> perm(n), iperm(n);
