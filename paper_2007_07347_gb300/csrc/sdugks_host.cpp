@@ -416,16 +416,28 @@ static int prepare(int prec, int kernel)
 static cudaError_t launch_one(sdugks_solver *s, cudaStream_t st)
 {
     const int a = s->cur;
+    const bool single = st != s->cap_stream;          // not into a graph: see early_start
     cudaError_t e;
     if (s->strip_rows > 0)
-        e = launch_step_strip(s->strip, s->strip_rows, s->strip_early, a, st);
-    else if (s->kernel == SDUGKS_KERNEL_CARTESIAN)
-        e = launch_step_cart(s->p.precision, s->launch_shape, s->ci, s->tma, s->cart_general, a, st);
-    else if (s->p.precision == P_FP64)
-        e = launch_step_tiled_fp64(s->tm, s->coefs, s->st.f[a], s->st.f[1 - a], s->st.W[a], s->st.W[1 - a], st);
-    else
-        e = launch_step_tiled_fp32(s->p.precision, s->tm, s->coefs, s->st.f[a], s->st.f[1 - a], s->st.W[a],
-                                   s->st.W[1 - a], st);
+        e = launch_step_strip(s->strip, s->strip_rows, s->strip_early || single, a, st);
+    else if (s->kernel == SDUGKS_KERNEL_CARTESIAN) {
+        CartInst ci = s->ci;
+        int shape = s->launch_shape;
+        if (single && !ci.early) {
+            // the blocks of the graph's step, smaller for being placed evenly, pile up: 200^2
+            // 5.4 us, with the general model's 5.0
+            ci.early = 1;
+            if (s->p.precision == P_FP32) shape = s->cart_shape;
+        }
+        e = launch_step_cart(s->p.precision, shape, ci, s->tma, s->cart_general, a, st);
+    } else {
+        TiledMesh tm = s->tm;
+        tm.early = tm.early || single;
+        e = s->p.precision == P_FP64
+                ? launch_step_tiled_fp64(tm, s->coefs, s->st.f[a], s->st.f[1 - a], s->st.W[a], s->st.W[1 - a], st)
+                : launch_step_tiled_fp32(s->p.precision, tm, s->coefs, s->st.f[a], s->st.f[1 - a], s->st.W[a],
+                                         s->st.W[1 - a], st);
+    }
     s->cur = 1 - a;
     return e;
 }
@@ -1910,7 +1922,7 @@ static cudaError_t batch_launch_step(const sdugks_batch *b, int parity, bool per
     cudaError_t e = cudaSuccess;
     for (const auto &g : b->groups)
         if (e == cudaSuccess)
-            e = launch_strip_batch(g.g, b->d_sitems + g.first, (int)g.n, b->strip_rows, b->strip_early, parity, st);
+            e = launch_strip_batch(g.g, b->d_sitems + g.first, (int)g.n, b->strip_rows, b->strip_early || st != b->cap_stream, parity, st);
     if (e == cudaSuccess && (b->n_block > 0 || b->groups.empty()))
         e = launch_step_batch(b->prec, b->d_inst, b->d_items, b->d_nitems + 1, grid, per_item, parity, st);
     return e;

@@ -226,13 +226,16 @@ cudaError_t launch_step_tiled_fp32(int prec, const TiledMesh &m, const Coefs &c,
 // next step's CTAs therefore take the SM slots the moment the current step's CTAs
 // retire, instead of after the launch latency.
 //
-// The early start suits grids that fill the device (at least 4/5 of its `slots` resident
-// CTAs), whose next CTAs take over slot by slot, and grids of a few CTAs.  In between, the next step's CTAs are placed while the current ones still run,
-// wherever there is room, and pile up on some SMs: the step then lasts as long as the
-// fullest SM.  GB300, us per step with / without: 169 tiles 8.2 / 6.1, 361 tiles 8.3 / 7.6,
-// 4x1024 channel (128 blocks) 4.1 / 3.6, 128^2 cavity 4.3 / 3.7; but 256^2 (304 blocks in 304
-// slots) 4.46 / 4.65, 1024 tiles in 608 slots 13.3 / 14.0, 4x256 channel (19 blocks) 3.44 / 3.53.
-inline bool early_start(int64_t ctas, int64_t slots, int n_sm) { return 4 * ctas <= n_sm || 5 * ctas >= 4 * slots; }
+// The early start suits grids whose fullest SM holds as many CTAs as fit anyway (more than
+// all SMs' slots but one each), whose next CTAs take over slot by slot, and grids of a few CTAs.
+// In between, the next step's CTAs are placed while the current ones still run, wherever there
+// is room, and pile up on some SMs: the step then lasts as long as the fullest SM.  GB300, us
+// per step with / without: 169 tiles of 608 slots 8.2 / 6.1, 441 tiles 8.45 / 8.07, 484 tiles 8.2 / 8.75,
+// 1024 tiles 13.3 / 14.0; 4x1024 channel (128 blocks of 608) 4.1 / 3.1, 4x256 channel (19 blocks)
+// 3.44 / 3.53; bf16 cavities of 144 blocks in 304 slots 4.52 / 4.46, 169 blocks 4.49 / 4.59, 196 blocks
+// 4.50 / 4.68.  These are steps of a graph.  Launched one by one, a step without the early start takes
+// 6.2 us at least (361 tiles 10.3), and with it 4.1 (8.8): it then always has it.
+inline bool early_start(int64_t ctas, int64_t slots, int n_sm) { return 4 * ctas <= n_sm || ctas > slots - n_sm; }
 
 #ifdef __CUDACC__
 __device__ __forceinline__ void step_dependency_wait()
