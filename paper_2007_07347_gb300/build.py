@@ -33,6 +33,7 @@ CU_UNITS = {
     "k_residual_noalloc.cu": [],
     "k_batch.cu": [],
     "k_dvm.cu": [],
+    "k_dvm_cart.cu": [],
 }
 CXX_UNITS = ["sdugks_host.cpp"]
 HEADERS = ["sdugks_internal.h", "d2q9.cuh", "step_tiled.cuh", "step_cart.cuh", "step_strip.cuh"]

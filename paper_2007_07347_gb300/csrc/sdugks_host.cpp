@@ -2323,7 +2323,86 @@ struct sdugks_dvm {
     int graph_len = 0;
     bool initialised = false;
     bool fbp_ready = false;         // fbp holds fbar+ of the current state (left by the last step)
+    // uniform Cartesian grids (k_dvm_cart.cu): two f buffers
+    bool cart = false;
+    DvmCart dc{};
+    DvmCartState ds{};
+    int cur = 0;
 };
+
+// Tables of the Cartesian rarefied step: constants, reference Maxwellian and walls.
+// m0, wt: factors of the reference and of the walls' Maxwellians in the compute precision.
+static void fill_dvm_cart(DvmCart &k, const sdugks_mesh &m, const CartGrid &g, const sdugks_dvm_params &prm,
+                          const std::vector<double> &node, std::vector<double> &m0, std::vector<double> &wt)
+{
+    const int nv = prm.nv;
+    const double h = 2.0 * prm.vmax / nv, RT = prm.RT_wall, pi = 3.14159265358979323846, tau = prm.tau, dt = prm.dt;
+    auto rnd = [&](double v) { return prm.precision == SDUGKS_FP64 ? v : (double)(float)v; };
+    std::vector<double> x(nv);
+    for (int j = 0; j < nv; j++) x[j] = rnd(node[j]);
+    auto factors = [&](double *t, double ux, double uy) {
+        for (int j = 0; j < nv; j++) {
+            t[j] = rnd(std::exp(-(node[j] - ux) * (node[j] - ux) / (2.0 * RT)));
+            t[nv + j] = rnd(h * h / (2.0 * pi * RT) * std::exp(-(node[j] - uy) * (node[j] - uy) / (2.0 * RT)));
+        }
+    };
+    m0.assign(2 * nv, 0.0);
+    wt.assign(8 * nv, 0.0);
+    factors(m0.data(), 0.0, 0.0);
+    DvmCartK<double> &d = k.kd;
+    d.w_node = h * h;
+    d.a = (2.0 * tau - dt) / (2.0 * tau); d.b = dt / (2.0 * tau); d.c = 2.0 * tau / (2.0 * tau + dt); d.cb = d.c * d.b;
+    d.r = dt / tau; d.inv1r = 1.0 / (1.0 + dt / tau); d.dtV = dt / (g.dx * g.dy);
+    d.len[0] = g.dy; d.len[1] = g.dx;
+    d.kh[0] = d.kh[1] = 0.25;                       // (h / 2) / (2 h)
+    d.kdt[0] = dt / (2.0 * g.dx); d.kdt[1] = dt / (2.0 * g.dy);
+    // half-range sums of one axis (the zero node of an odd grid in both halves, by half)
+    auto half = [&](const double *t, int pos, int pw) {
+        double s = 0.0;
+        for (int j = 0; j < nv; j++) {
+            const bool zero = nv % 2 && j == nv / 2;
+            if (!zero && (j >= nv / 2) != (pos != 0)) continue;
+            s += (zero ? 0.5 : 1.0) * t[j] * std::pow(x[j], pw);
+        }
+        return s;
+    };
+    for (int n = 0; n <= 4; n++)
+        for (int b = 0; b <= n; b++) {
+            const int i = n * (n + 1) / 2 + b;
+            d.m0f[i] = 0.0;
+            for (int q = 0; q < 4; q++) {
+                d.m0f[i] += half(m0.data(), q & 1, n - b) * half(m0.data() + nv, q >> 1, b);
+            }
+        }
+    for (int q = 0; q < 2; q++)
+        for (int b = 0; b < 2; b++) d.m0s[q][b] = half(m0.data() + q * nv, 0, 2 * b) + half(m0.data() + q * nv, 1, 2 * b);
+    // walls in the order E, W, N, S
+    const int side_of[4] = {1, 3, 2, 0};
+    for (int w = 0; w < 4; w++) {
+        DvmWall &wl = k.wall[w];
+        std::memset(&wl, 0, sizeof wl);
+        const int32_t p = g.side_patch[side_of[w]];
+        const bool moving = m.bc_kind[p] == SDUGKS_BC_MOVING_WALL;
+        double *t = wt.data() + (size_t)w * 2 * nv;
+        factors(t, moving ? m.bc_par[p][0] : 0.0, moving ? m.bc_par[p][1] : 0.0);
+        for (int i = 0; i < nv; i++)
+            for (int j = 0; j < nv; j++) {
+                const double s = w == 0 ? x[j] : w == 1 ? -x[j] : w == 2 ? x[i] : -x[i];
+                const double psi[4] = {1.0, x[j], x[i], 0.5 * (x[j] * x[j] + x[i] * x[i])};
+                const double gg = t[j] * t[nv + i], mm = m0[j] * m0[nv + i];
+                for (int q = 0; q < 4; q++) {
+                    (s < 0.0 ? wl.g_in : wl.g_out)[q] += s * psi[q] * gg;
+                    (s < 0.0 ? wl.m0_in : wl.m0_out)[q] += s * psi[q] * mm;
+                }
+            }
+    }
+    DvmCartK<float> &f = k.kf;
+    f.w_node = (float)d.w_node; f.a = (float)d.a; f.b = (float)d.b; f.c = (float)d.c; f.cb = (float)d.cb; f.r = (float)d.r;
+    f.inv1r = (float)d.inv1r; f.dtV = (float)d.dtV;
+    for (int q = 0; q < 2; q++) { f.len[q] = (float)d.len[q]; f.kh[q] = (float)d.kh[q]; f.kdt[q] = (float)d.kdt[q]; }
+    for (int q = 0; q < 15; q++) f.m0f[q] = (float)d.m0f[q];
+    for (int q = 0; q < 4; q++) f.m0s[q / 2][q % 2] = (float)d.m0s[q / 2][q % 2];
+}
 
 extern "C" int sdugks_dvm_create(const sdugks_mesh *m, const sdugks_dvm_params *prm, void *stream, sdugks_dvm **out)
 {
@@ -2415,16 +2494,54 @@ extern "C" int sdugks_dvm_create(const sdugks_mesh *m, const sdugks_dvm_params *
     std::vector<double> vn(prm->nv);
     for (int j = 0; j < prm->nv; j++) vn[j] = -prm->vmax + (j + 0.5) * h;
 
+    // uniform Cartesian grids take their own step (k_dvm_cart.cu)
+    CartGrid grid;
+    const bool cart = prm->dt <= prm->tau && detect_cart(*m, grid) && dvm_cart_fits(prm->precision == SDUGKS_FP64 ? P_FP64 : P_FP32, n, prm->nv, grid.ny);
+    DvmCart dc{};
+    std::vector<double> m0, wt;
+    std::vector<int32_t> nbt, at;
+    if (cart) {
+        fill_dvm_cart(dc, *m, grid, *prm, vn, m0, wt);
+        at.resize(n);
+        for (int64_t c = 0; c < n; c++) at[grid.ci[c] + (int64_t)grid.nx * grid.cj[c]] = (int32_t)c;
+        nbt.resize(4 * (size_t)n);
+        const int di[4] = {1, -1, 0, 0}, dj[4] = {0, 0, 1, -1};
+        for (int64_t c = 0; c < n; c++)
+            for (int w = 0; w < 4; w++) {
+                int i = grid.ci[c] + di[w], j = grid.cj[c] + dj[w];
+                if (grid.px) i = (i + grid.nx) % grid.nx;
+                if (grid.py) j = (j + grid.ny) % grid.ny;
+                nbt[4 * (size_t)c + w] = i < 0 || i >= grid.nx || j < 0 || j >= grid.ny ? -1 : at[i + (int64_t)grid.nx * j];
+            }
+    }
+
     sdugks_dvm *d = new (std::nothrow) sdugks_dvm;
     if (!d) return fail(SDUGKS_ERR_OOM, "host allocation failed");
     d->p = *prm;
     if (d->p.graph_steps == 0) d->p.graph_steps = 32;
+    if (cart && d->p.graph_steps > 0) d->p.graph_steps = std::max(2, d->p.graph_steps / 2 * 2);   // two f buffers
+    d->cart = cart;
+    d->dc = dc;
     d->prec = prm->precision;
     d->rs = d->prec == P_FP64 ? 8 : 4;
     d->stream = static_cast<cudaStream_t>(stream);
     d->n = n; d->nf = nf; d->Q = Q;
     const size_t rs = d->rs;
+    const size_t nv = (size_t)prm->nv;
     auto layout = [&](Arena &A) {
+        if (cart) {
+            for (int b = 0; b < 2; b++) d->ds.phi[b] = A.take<char>((size_t)n * Q * rs);
+            for (int b = 0; b < 2; b++) d->ds.tab[b] = A.take<char>((size_t)n * dvm_cart_table(prm->nv) * rs);
+            d->ds.mom = A.take<char>((size_t)n * 60 * rs);
+            d->ds.face_tab = A.take<char>((size_t)n * 4 * dvm_cart_table(prm->nv) * rs);
+            d->ds.W = d->W = A.take<double>((size_t)n * 4);
+            d->dc.nb = A.take<int32_t>(nbt.size());
+            d->dc.at = A.take<int32_t>(at.size());
+            d->dc.vnode = A.take<char>(nv * rs);
+            d->dc.m0 = A.take<char>(2 * nv * rs);
+            d->dc.wall_tab = A.take<char>(8 * nv * rs);
+            return;
+        }
         d->f = A.take<char>((size_t)n * Q * rs);
         d->fbp = A.take<char>((size_t)n * Q * rs);
         d->flux = A.take<char>((size_t)nf * Q * rs);
@@ -2469,6 +2586,24 @@ extern "C" int sdugks_dvm_create(const sdugks_mesh *m, const sdugks_dvm_params *
         if (ee != cudaSuccess && rc2 == SDUGKS_OK) rc2 = fail(SDUGKS_ERR_CUDA, "%s: %s", what, cudaGetErrorString(ee));
     };
     const auto gcd = conv(cd), gai = conv(ainv), gfg = conv(fgeo), gvn = conv(vn);
+    if (cart) {
+        const auto gm0 = conv(m0), gwt = conv(wt);
+        d->dc.nc = (int32_t)n; d->dc.nv = prm->nv; d->dc.Q = Q;
+        up(d->dc.nb, nbt.data(), nbt.size() * 4, "upload neighbours");
+        up(d->dc.at, at.data(), at.size() * 4, "upload lattice");
+        d->dc.nx = grid.nx; d->dc.ny = grid.ny; d->dc.per_x = grid.px; d->dc.per_y = grid.py;
+        up(d->dc.vnode, gvn.data(), gvn.size(), "upload velocity nodes");
+        up(d->dc.m0, gm0.data(), gm0.size(), "upload the reference");
+        up(d->dc.wall_tab, gwt.data(), gwt.size(), "upload wall tables");
+        if (rc2 == SDUGKS_OK) {
+            cudaError_t ee = cudaStreamCreateWithFlags(&d->cap_stream, cudaStreamNonBlocking);
+            if (ee == cudaSuccess) ee = prepare_dvm_cart(d->prec, d->dc);
+            if (ee != cudaSuccess) rc2 = fail(SDUGKS_ERR_CUDA, "stream / kernel attributes: %s", cudaGetErrorString(ee));
+        }
+        if (rc2) { sdugks_dvm_destroy(d); return rc2; }
+        *out = d;
+        return SDUGKS_OK;
+    }
     up(d->dm.cell_face, cface.data(), cface.size() * 4, "upload cell faces");
     up(d->dm.cell_nb, cnb.data(), cnb.size() * 4, "upload neighbours");
     up(d->dm.cell_d, gcd.data(), gcd.size(), "upload offsets");
@@ -2502,7 +2637,9 @@ extern "C" int sdugks_dvm_init(sdugks_dvm *d, const double *rho, const double *u
     }
     CUDA_TRY(cudaSetDevice(d->device));
     CUDA_TRY(cudaMemcpyAsync(d->W, W.data(), W.size() * 8, cudaMemcpyHostToDevice, d->stream));
-    CUDA_TRY(launch_dvm_init(d->prec, d->dm, d->W, d->f, d->stream));
+    d->cur = 0;
+    if (d->cart) CUDA_TRY(launch_dvm_cart_init(d->prec, d->dc, d->ds, d->stream));
+    else CUDA_TRY(launch_dvm_init(d->prec, d->dm, d->W, d->f, d->stream));
     CUDA_TRY(cudaStreamSynchronize(d->stream));
     d->initialised = true;
     d->fbp_ready = false;
@@ -2516,8 +2653,9 @@ static int dvm_ensure_graph(sdugks_dvm *d)
     cudaGraph_t g = nullptr;
     CUDA_TRY(cudaStreamBeginCapture(d->cap_stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
-    for (int k = 0; k < G && e == cudaSuccess; k++)     // replayed only once fbp is ready
-        e = launch_dvm_step(d->prec, d->dm, d->coefs, d->p.RT_wall, d->f, d->W, d->fbp, d->flux, true, d->cap_stream);
+    for (int k = 0; k < G && e == cudaSuccess; k++)     // replayed only once fbp is ready, from f buffer 0
+        if (d->cart) e = launch_dvm_cart_step(d->prec, d->dc, d->ds, k & 1, d->cap_stream);
+        else e = launch_dvm_step(d->prec, d->dm, d->coefs, d->p.RT_wall, d->f, d->W, d->fbp, d->flux, true, d->cap_stream);
     cudaError_t e2 = cudaStreamEndCapture(d->cap_stream, &g);
     CUDA_TRY(e);
     CUDA_TRY(e2);
@@ -2536,6 +2674,22 @@ extern "C" int sdugks_dvm_step(sdugks_dvm *d, int64_t n)
     CUDA_TRY(cudaSetDevice(d->device));
     int64_t left = n;
     const int G = d->p.graph_steps;
+    auto one = [&] {
+        const cudaError_t e = launch_dvm_cart_step(d->prec, d->dc, d->ds, d->cur, d->stream);
+        d->cur ^= 1;
+        left--;
+        return e;
+    };
+    if (d->cart) {
+        if (G > 0 && left > G && d->cur != 0) CUDA_TRY(one());
+        if (G > 0 && left >= G && d->cur == 0) {
+            int rc = dvm_ensure_graph(d);
+            if (rc) return rc;
+            for (; left >= G; left -= G) CUDA_TRY(cudaGraphLaunch(d->graph, d->stream));
+        }
+        while (left > 0) CUDA_TRY(one());
+        return SDUGKS_OK;
+    }
     if (left > 0 && !d->fbp_ready) {
         CUDA_TRY(launch_dvm_step(d->prec, d->dm, d->coefs, d->p.RT_wall, d->f, d->W, d->fbp, d->flux, false, d->stream));
         d->fbp_ready = true;
@@ -2574,11 +2728,14 @@ extern "C" int sdugks_dvm_get_state(sdugks_dvm *d, double *f, double *W)
     if (W) CUDA_TRY(cudaMemcpyAsync(W, d->W, (size_t)d->n * 4 * 8, cudaMemcpyDeviceToHost, d->stream));
     if (f) {
         const size_t cnt = (size_t)d->n * d->Q;
+        // the other buffer holds nothing between steps
+        if (d->cart) CUDA_TRY(launch_dvm_cart_f(d->prec, d->dc, d->ds, d->cur, d->stream));
+        const void *df = d->cart ? d->ds.phi[1 - d->cur] : d->f;
         if (d->prec == P_FP64) {
-            CUDA_TRY(cudaMemcpyAsync(f, d->f, cnt * 8, cudaMemcpyDeviceToHost, d->stream));
+            CUDA_TRY(cudaMemcpyAsync(f, df, cnt * 8, cudaMemcpyDeviceToHost, d->stream));
         } else {
             std::vector<float> tmp(cnt);
-            CUDA_TRY(cudaMemcpyAsync(tmp.data(), d->f, cnt * 4, cudaMemcpyDeviceToHost, d->stream));
+            CUDA_TRY(cudaMemcpyAsync(tmp.data(), df, cnt * 4, cudaMemcpyDeviceToHost, d->stream));
             CUDA_TRY(cudaStreamSynchronize(d->stream));
             for (size_t i = 0; i < cnt; i++) f[i] = tmp[i];
         }

@@ -289,6 +289,46 @@ cudaError_t launch_dvm_step(int prec, const DvmMesh &m, const Coefs &c, double R
 cudaError_t launch_dvm_init(int prec, const DvmMesh &m, const double *W, void *f, cudaStream_t st);
 cudaError_t prepare_dvm(int prec, int64_t Q, int nv);   // kernel attributes on the current device
 
+// Rarefied solver on a uniform Cartesian grid (k_dvm_cart.cu).  Sums over the leaving and
+// the entering velocities of a wall of xi_n (outward) times (1, x, y, (x^2 + y^2) / 2): of
+// the wall's Maxwellian of unit density (g) and of the reference (m0).
+struct DvmWall {
+    double g_out[4], g_in[4], m0_out[4], m0_in[4];
+};
+template <class R> struct DvmCartK {
+    R w_node, a, b, c, cb, r, inv1r, dtV;
+    R len[2];                  // length of a face of constant x, y
+    R kh[2], kdt[2];           // h / 2 and dt along x and y, times 1 / (2 h)
+    R m0f[15], m0s[2][2];      // moments of the reference; of its factors along x and y (powers 0 and 2)
+};
+struct DvmCart {
+    int32_t nc, nv, nx, ny, per_x, per_y;
+    int32_t chunks, seg;       // the update: CTAs per line and quadrant, cells of a line per CTA
+    int64_t Q;
+    const int32_t *at;         // [ny][nx] cell of a lattice position
+    const int32_t *nb;         // [nc][4] neighbour E, W, N, S; -1 a wall
+    const void *vnode;         // [nv] nodes of one axis (compute precision)
+    const void *m0;            // [2][nv] factors of the reference Maxwellian (x; y with the node weight)
+    const void *wall_tab;      // [4][2][nv] factors of the wall Maxwellians of the E, W, N, S sides
+    DvmCartK<double> kd;
+    DvmCartK<float> kf;
+    DvmWall wall[4];
+};
+struct DvmCartState {
+    void *phi[2];              // [nc][Q] fbar+
+    double *W;                 // [nc][4]
+    void *tab[2];              // [nc][table] factors of feq(W)
+    void *mom;                 // [nc][4][15] quadrant moments of fbar+
+    void *face_tab;            // [nc][4][table] factors of the interface equilibria
+};
+bool dvm_cart_fits(int prec, int64_t nc, int nv, int ny);
+size_t dvm_cart_table(int nv);          // values of one table
+cudaError_t prepare_dvm_cart(int prec, DvmCart &m);
+cudaError_t launch_dvm_cart_init(int prec, const DvmCart &m, const DvmCartState &s, cudaStream_t st);
+// f of the state in phi[parity], into the other buffer
+cudaError_t launch_dvm_cart_f(int prec, const DvmCart &m, const DvmCartState &s, int parity, cudaStream_t st);
+cudaError_t launch_dvm_cart_step(int prec, const DvmCart &m, const DvmCartState &s, int parity, cudaStream_t st);
+
 // state conversions between the caller's cell-major FP64 layout (user cell order)
 // and the internal SoA layout: the q-th listed cell is user cell perm[q] stored at
 // internal offset loc[q] (loc == nullptr: offset q).
