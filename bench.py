@@ -213,7 +213,7 @@ def measured_peaks():
 STEP_SOURCES = {
     "k_step_cart": ["d2q9.cuh", "sdugks_internal.h", "step_cart.cuh", "k_cart.cu"],
     "k_step_tiled": ["d2q9.cuh", "sdugks_internal.h", "step_tiled.cuh", "k_step_fp32.cu"],
-    "k_step_batch": ["d2q9.cuh", "sdugks_internal.h", "step_cart.cuh", "k_batch.cu"],
+    "k_strip_batch": ["d2q9.cuh", "sdugks_internal.h", "step_strip.cuh", "k_strip.cu"],
 }
 
 
@@ -355,6 +355,8 @@ def roofline_of(info, precision, n, launch_ms, key):
     alg_bytes = (STATE_BYTES[precision] + mesh_b) * n
     achieved = alg_bytes / (launch_ms / 1e3) / 1e9
     kname = {1: "k_step_tiled", 2: "k_step_cart"}[info["kernel"]]
+    if kname == "k_step_cart" and precision == "fp32" and n >= 448 * 448:
+        kname = "k_step_strip"           # large FP32 grids march
     resident = (STATE_BYTES[precision] + mesh_b) * n < 0.8 * L2_BYTES
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "traffic": profiled_traffic(key), "kernel": kname, "algorithmic_bytes_per_launch": alg_bytes,
@@ -511,12 +513,12 @@ def other_configs(args, S, stream, flush):
     launch_s = t / (interval * bsteps)               # the residual reductions are included
     out["batch_256_cavities_fp32"] = {
         "workload": "batch of 256 lid-driven cavities, N~logU[32,512], Re~logU[100,5000], seed 1, lid 0.1, CFL 0.5, "
-                    "FP32, one batched launch per step over the (instance, 16x8 block) work list",
+                    "FP32, one batched launch per step over the (instance, strip of columns, rows) work list",
         "value": cells * 9 * interval * bsteps / t / 1e6, "unit": "MLUPS", "steps": bsteps,
         "time_steps_per_step": interval, "ms_per_step": 1e3 * t / bsteps, "cells": cells,
         "roofline": {"bound": "hbm", "achieved": alg / launch_s / 1e9, "peak": peak, "unit": "GB/s",
-                     "frac": alg / launch_s / 1e9 / peak, "traffic": profiled_traffic("k_step_batch_fp32_batch256"),
-                     "kernel": "k_step_batch",
+                     "frac": alg / launch_s / 1e9 / peak, "traffic": profiled_traffic("k_strip_batch_fp32_batch256"),
+                     "kernel": "k_strip_batch",
                      "algorithmic_bytes_per_launch": alg, "avg_launch_us": launch_s * 1e6,
                      "peak_kind": f"{peak_kind} (hbm_gbs)", "l2_resident": False,
                      "note": "1.4 GB of state: every launch streams it from HBM; the launch time includes the share "
@@ -769,9 +771,8 @@ def run_serve(args):
 
 def run_rarefied(args):
     """Micro cavity of Sec. IV: 40 x 40 cells, 100 x 100 velocities on [-2, 2]^2, Kn = 1,
-    diffuse walls, lid 0.1, FP32 f.  One benchmark step = 200 time steps (2 launches
-    each, face and cell kernels, graphs of 32 steps; the cell kernel leaves the next
-    step's fbar+).  MLUPS counts cell-velocity updates (Q = 10^4)."""
+    diffuse walls, lid 0.1, FP32 f.  One benchmark step = 200 time steps (3 launches
+    each: moments, interface states, update; graphs of 32 steps).  MLUPS counts cell-velocity updates (Q = 10^4)."""
     import torch
     from paper_2007_07347_gb300 import sdugks as S
     torch.cuda.set_device(0)
@@ -780,7 +781,7 @@ def run_rarefied(args):
     stream = torch.cuda.Stream()
     d = S.Dvm.from_case(case, prec, stream=stream).init()
     sz = d.sizes()
-    n, Q, nf = sz["n_cells"], sz["Q"], sz["n_faces"]
+    n, Q = sz["n_cells"], sz["Q"]
     interval = 200
     flush = torch.empty(256 * 1024 * 1024 // 4, dtype=torch.float32, device="cuda")
     with torch.cuda.stream(stream):
@@ -801,7 +802,7 @@ def run_rarefied(args):
     step_s = tot_s / (interval * args.steps)
     rs = 8 if prec == "fp64" else 4
     alg = n * Q * 2 * rs + n * 4 * 8 * 2              # f read and written once, W read and written
-    scratch = (n * Q * 2 + nf * Q * 3) * rs            # fbar+ (write, read) and face fluxes (write, read twice)
+    scratch = 4 * n * Q * rs                           # fbar+ read once for its moments, four times by the march
     peak, peak_kind = measured_peaks()
     # e2e: through the C-ABI, the macroscopic state read back to the host every benchmark step
     t0 = time.perf_counter()
@@ -833,16 +834,16 @@ def run_rarefied(args):
             "config": {"workload": "rarefied micro cavity 40x40, 100x100 velocities on [-2,2]^2, Kn 1, lid 0.1, "
                                    "diffuse walls", "cells": n, "velocities": Q, "time_steps_per_step": interval,
                        "storage": prec, "tau": case.tau, "dt": case.dt,
-                       "l2": "flushed (256 MB rewrite) before each timed step; f, fbar+ and the face fluxes "
-                             f"({(2 * n + nf) * Q * rs / 1e6:.0f} MB) exceed L2"},
+                       "l2": "flushed (256 MB rewrite) before each timed step; the two buffers of fbar+ "
+                             f"({2 * n * Q * rs / 1e6:.0f} MB) about fill L2"},
             "roofline": {"bound": "hbm", "achieved": alg / step_s / 1e9, "peak": peak, "unit": "GB/s",
                          "frac": alg / step_s / 1e9 / peak, "traffic": None,
-                         "kernel": "one time step (k_dvm_face + k_dvm_cell)",
+                         "kernel": "one time step (k_dvc_moments + k_dvc_states + k_dvc_update)",
                          "algorithmic_bytes_per_launch": alg, "scratch_bytes_per_step": scratch,
                          "avg_step_us": step_s * 1e6, "peak_kind": f"{peak_kind} (hbm_gbs)"},
             "e2e": {"value": n * Q * interval * e2e_steps / e2e_s / 1e6, "unit": "MLUPS", "h2d_bytes_per_step": 0,
                     "d2h_bytes_per_step": n * 4 * 8},
-            "gpu_launches": 2 * interval * args.steps,
+            "gpu_launches": 3 * interval * args.steps,
             "max_u_over_lid": float(np.abs(u).max() / 0.1), "mass": float(rho.sum())}
     clocks = clk.summary()
     if clocks:

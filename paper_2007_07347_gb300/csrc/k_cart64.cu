@@ -349,8 +349,8 @@ template <int BX, int BY> cudaError_t launch64(const CartInst &m, int parity, cu
 {
     using Sh = Shape64<BX, BY>;
     const dim3 grid((m.nx + BX - 1) / BX, (m.ny + BY - 1) / BY);
-    // no early start: the blocks have to lie evenly on the SMs' FP64 pipes (256^2: 62.8 us, with
-    // it 87.3)
+    // no early start: the blocks have to lie evenly on the SMs' FP64 pipes (256^2, in this kernel's
+    // first form: 62.8 us, with it 87.3; now 54)
     if (m.force || m.bface)
         return launch_step_kernel(false, k_step_cart64<BX, BY, true>, grid, dim3(Sh::NT), Sh::SMEM, st, m, coefs64(m), parity);
     return launch_step_kernel(false, k_step_cart64<BX, BY, false>, grid, dim3(Sh::NT), Sh::SMEM, st, m, coefs64(m), parity);

@@ -6,7 +6,7 @@ CASE is one of cavity128, cavity256, cavity1024, cylinder (512 x 256 O-mesh),
 microcavity (the rarefied solver: 40 x 40 cells, 100 x 100 velocities, Kn 1), batch
 (the 256 cavities of the batched configuration, N ~ logU[32, 512], seed 1) or batchK
 (the first K of those 256, e.g. batch32 for a capture that holds less device memory).  Used
-under ncu with ``-k regex:k_step`` (``regex:k_dvm`` for the rarefied kernels) to
+under ncu with ``-k regex:k_step`` (``regex:k_strip`` for FP32 batches, ``regex:k_dv`` for the rarefied kernels) to
 capture single step launches.  STAGING (Cartesian kernel): loads (default) or tma.
 """
 import sys
