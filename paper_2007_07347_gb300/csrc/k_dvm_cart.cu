@@ -47,16 +47,17 @@ template <class R> __device__ __forceinline__ const DvmCartK<R> &consts(const Dv
 template <> __device__ __forceinline__ const DvmCartK<float> &consts<float>(const DvmCart &m) { return m.kf; }
 template <> __device__ __forceinline__ const DvmCartK<double> &consts<double>(const DvmCart &m) { return m.kd; }
 
-// exp(-(x - u)^2 beta); FP32: beta times log2 e.  In FP32 to about half an ulp: the rounding errors of the
+// exp(-(x - u)^2 beta); FP32: beta times log2 e.  In FP32 to about one ulp: the rounding errors of the
 // difference and of the products are carried along, and 2^r on |r| <= 1/2 is its Taylor
 // series (the term of degree 8 is below 6e-9): the errors of a table of nv nodes average out less than
-// those of nv^2 Maxwellians would.
+// those of nv^2 Maxwellians would.  A run that breaks down (R T, and with it beta, below zero) has to
+// show it: the exponential's overflow is infinity and an undefined exponent NaN, as exp gives them.
 template <class R> __device__ __forceinline__ R gauss(R x, R u, R beta);
 template <> __device__ __forceinline__ float gauss<float>(float x, float u, float beta)
 {
     const float d = x - u, v = d - x, dl = (x - (d - v)) + (-u - v);
     const float hi = d * d, lo = fmaf(d, d, -hi) + 2.0f * d * dl, t = hi * beta, tl = fmaf(hi, beta, -t) + lo * beta;
-    const float n = rintf(fminf(t, 140.0f)), r = n - t;                   // 2^-t = 2^-n 2^r
+    const float n = rintf(fmaxf(fminf(t, 140.0f), -128.0f)), r = n - t;   // 2^-t = 2^-n 2^r
     float q = 1.5252734e-5f;                                              // (ln 2)^k / k!, k = 7 .. 1
     q = fmaf(q, r, 1.5403530e-4f);
     q = fmaf(q, r, 1.3333558e-3f);
@@ -65,6 +66,7 @@ template <> __device__ __forceinline__ float gauss<float>(float x, float u, floa
     q = fmaf(q, r, 2.4022651e-1f);
     q = fmaf(q, r, 6.9314718e-1f);
     const float g = 1.0f + fmaf(q, r, -0.69314718f * tl * fmaf(q, r, 1.0f));
+    if (!(t > -128.0f)) return t != t ? t : INFINITY;
     return t < 120.0f ? g * __int_as_float((127 - (int)n) << 23) : 0.0f;
 }
 template <> __device__ __forceinline__ double gauss<double>(double x, double u, double beta) { return exp(-(x - u) * (x - u) * beta); }

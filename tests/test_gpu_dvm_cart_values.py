@@ -1,0 +1,55 @@
+"""Values of the rarefied step on uniform grids (k_dvm_cart.cu) that agreement over a few
+steps does not show: the Maxwellian's exponential over its whole range, and errors that grow
+with the number of steps."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2007_07347_gb300 import meshes as M
+
+pytestmark = pytest.mark.gpu
+
+
+def _S():
+    from paper_2007_07347_gb300 import sdugks as S
+    return S
+
+
+def test_initial_maxwellian_to_rounding():
+    """f of the initial state, rho = 1, u = 0, R T = 1/2 on nodes that FP32 holds exactly.  A
+    value is the product of two exponentials and a factor.  In units of 2^-23: two exponentials
+    of up to 1.5 each; the factor, 1 for its constant and product and 0.5 for its product with an
+    exponential; 0.5 for the last product; and log2 e rounded, 1.4e-8 of an exponent of up to 8, 1:
+    6 in all."""
+    S = _S()
+    n, nv = 10, 64
+    c = M.micro_cavity(n, 1.0, nv=nv)
+    d = S.Dvm.from_case(c, "fp32").init()
+    f = d.get_state()[0].reshape(n * n, nv, nv)
+    x = -2.0 + (np.arange(nv) + 0.5) * (4.0 / nv)
+    g = (4.0 / nv) ** 2 / np.pi * np.exp(-(x[None, :] ** 2 + x[:, None] ** 2))
+    assert np.abs(f / g - 1.0).max() <= 6 * 2.0 ** -23
+
+
+@pytest.mark.parametrize("seed", [5, 15, 17])
+def test_a_breakdown_does_not_read_as_finite(seed):
+    """One step of two cells from a noisy state leaves cells with R T < 0.  In those between -0.02
+    and -0.001 one of the outermost nodes, at +-1.97, has an exponent of at least 139 in base 2 for any
+    u: the Maxwellian overflows, and f, the only sign of a breakdown that this solver
+    gives, is not finite."""
+    S = _S()
+    n, nv = 10, 64
+    c = M.micro_cavity(n, 1.0, nv=nv)
+    rng = np.random.default_rng(seed)
+    rho, u = np.exp(rng.uniform(-0.8, 0, n * n)), rng.uniform(-0.1, 0.1, (n * n, 2))
+    RT, dt = 0.5 * np.exp(rng.uniform(-2, 0, n * n)), 4 * c.dt
+    tau = max(c.tau, dt)
+    d = S.Dvm(S.Mesh(c.mesh, c.bcs), nv, 2.0, 0.5, tau, dt, "fp32").init(rho, u, RT)
+    d.step(1)
+    xi, w = O.dvm_grid(nv, 2.0)
+    st = O.dvm_init(n * n, xi, w, rho=rho, u=u, RT=RT, RT0=0.5)
+    O.dvm_run(c.mesh, c.bcs, st, xi, w, 0.5, tau, dt, 1)
+    cold = np.where((st.RT > -0.02) & (st.RT < -0.001))[0]
+    f = d.get_state()[0]
+    assert len(cold) and not any(np.isfinite(f[i]).all() for i in cold)
+
