@@ -401,24 +401,23 @@ __global__ void __launch_bounds__(STATE_THREADS) k_dvc_states(const DvmCart m, c
                 flux[w][3] = to_f64<R>(sg * (R(0.5) * (d[6] + d[7]) + bb * f4));
             }
         } else {
-            // diffuse wall (Sec. III) on this side: rho_w so that no mass passes.  The
-            // wall's sums of xi_n (outward) times (1, x, y, e) over the leaving and entering
-            // velocities: of its Maxwellian g, and of the reference
+            // diffuse wall (Sec. III) on this side: rho_w = 1 + dw so that no mass passes.  The
+            // flux is the reference's share (DvmWall.z) plus c times what leaves of fbar beyond
+            // the reference and dw's: small terms, whose rounding, alike in every step, adds
+            // up to little (taken as the difference of whole fluxes, it put u off by 7e-14)
             const DvmWall &wl = m.wall[w];
             const R sg = out ? R(1) : R(-1);
-            const double so = wl.m0_out[0] + double(sg * d[1]);
-            const double rw = -m.kd.c * so / (m.kd.cb * wl.g_out[0] + wl.g_in[0]);
+            const double dw = -(wl.rest + double(sg * d[1])) / wl.g[0];
             const R *gw = static_cast<const R *>(m.wall_tab) + (int64_t)w * 2 * nv;
             for (int j = lane; j < nv; j += 32) {
                 ft[j] = gw[j];
-                ft[tab_row(nv, j)] = (R)(rw * (double)gw[nv + j]);
+                const double gy = (double)gw[nv + j];
+                ft[tab_row(nv, j)] = (R)fma(dw, gy, gy);
             }
             if (lane < 4) {
                 const R dn = d[3], dt_ = d[4];
                 const R o = lane == 0 ? d[1] : lane == 3 ? R(0.5) * (d[6] + d[7]) : ((lane == 1) == (ax == 0) ? dn : dt_);
-                flux[w][lane] = m.kd.len[ax] * (m.kd.c * (wl.m0_out[lane] + double(sg * o)) +
-                                             rw * (m.kd.cb * wl.g_out[lane] + wl.g_in[lane]) -
-                                             (wl.m0_out[lane] + wl.m0_in[lane]));
+                flux[w][lane] = lane == 0 ? 0.0 : m.kd.len[ax] * (wl.z[lane] + m.kd.c * (double(sg * o) + dw * wl.g[lane]));
             }
         }
     }

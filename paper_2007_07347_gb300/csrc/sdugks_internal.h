@@ -289,14 +289,17 @@ cudaError_t launch_dvm_step(int prec, const DvmMesh &m, const Coefs &c, double R
 cudaError_t launch_dvm_init(int prec, const DvmMesh &m, const double *W, void *f, cudaStream_t st);
 cudaError_t prepare_dvm(int prec, int64_t Q, int nv);   // kernel attributes on the current device
 
-// Rarefied solver on a uniform Cartesian grid (k_dvm_cart.cu).  Sums over the leaving and
-// the entering velocities of a wall of xi_n (outward) times (1, x, y, (x^2 + y^2) / 2): of
-// the wall's Maxwellian of unit density (g) and of the reference (m0).
+// Rarefied solver on a uniform Cartesian grid (k_dvm_cart.cu).  A wall, from sums of xi_n
+// (outward) times (1, x, y, (x^2 + y^2) / 2), with 1 + b = 1 / c:
 struct DvmWall {
-    double g_out[4], g_in[4], m0_out[4], m0_in[4];
+    double g[4];               // of its Maxwellian of unit density: b times over the leaving velocities plus
+                               // 1 + b times over the entering ones
+    double rest;               // g[0] plus the mass that leaves in the reference Maxwellian
+    double z[4];               // c (leaving part of the reference + g) less the whole reference: the flux,
+                               // less the reference's, for a cell that holds the reference
 };
 template <class R> struct DvmCartK {
-    R w_node, a, b, c, cb, r, inv1r, dtV;
+    R w_node, a, b, c, r, inv1r, dtV;
     R len[2];                  // length of a face of constant x, y
     R kh[2], kdt[2];           // h / 2 and dt along x and y, times 1 / (2 h)
     R m0f[15], m0s[2][2];      // moments of the reference; of its factors along x and y (powers 0 and 2)
