@@ -52,11 +52,13 @@ template <> __device__ __forceinline__ const DvmCartK<double> &consts<double>(co
 // series (the term of degree 8 is below 6e-9): the errors of a table of nv nodes average out less than
 // those of nv^2 Maxwellians would.  A run that breaks down (R T, and with it beta, below zero) has to
 // show it: the exponential's overflow is infinity and an undefined exponent NaN, as exp gives them.
-template <class R> __device__ __forceinline__ R gauss(R x, R u, R beta);
-template <> __device__ __forceinline__ float gauss<float>(float x, float u, float beta)
+// ul, bl: what u and beta leave out (FP32).
+template <class R> __device__ __forceinline__ R gauss(R x, R u, R beta, R ul = R(0), R bl = R(0));
+template <> __device__ __forceinline__ float gauss<float>(float x, float u, float beta, float ul, float bl)
 {
-    const float d = x - u, v = d - x, dl = (x - (d - v)) + (-u - v);
-    const float hi = d * d, lo = fmaf(d, d, -hi) + 2.0f * d * dl, t = hi * beta, tl = fmaf(hi, beta, -t) + lo * beta;
+    const float d = x - u, v = d - x, dl = (x - (d - v)) + (-u - v) - ul;
+    const float hi = d * d, lo = fmaf(d, d, -hi) + 2.0f * d * dl, t = hi * beta;
+    const float tl = fmaf(hi, beta, -t) + fmaf(lo, beta, hi * bl);
     const float n = rintf(fmaxf(fminf(t, 140.0f), -128.0f)), r = n - t;   // 2^-t = 2^-n 2^r
     float q = 1.5252734e-5f;                                              // (ln 2)^k / k!, k = 7 .. 1
     q = fmaf(q, r, 1.5403530e-4f);
@@ -69,7 +71,10 @@ template <> __device__ __forceinline__ float gauss<float>(float x, float u, floa
     if (!(t > -128.0f)) return t != t ? t : INFINITY;
     return t < 120.0f ? g * __int_as_float((127 - (int)n) << 23) : 0.0f;
 }
-template <> __device__ __forceinline__ double gauss<double>(double x, double u, double beta) { return exp(-(x - u) * (x - u) * beta); }
+template <> __device__ __forceinline__ double gauss<double>(double x, double u, double beta, double, double)
+{
+    return exp(-(x - u) * (x - u) * beta);
+}
 
 // Pairs of velocities (two columns in the moments, two rows in the update): paired FP32
 // instructions, or two FP64 ones.
@@ -162,27 +167,74 @@ template <class R> __device__ __forceinline__ R half_sum(const R *t, const R *xp
     return s;
 }
 
-// Parameters of feq of a cell's W: {factor, ux, uy, beta}.
-template <class R>
-__device__ __forceinline__ void state_params(R par[4], double rho_d, double mx, double my, double rE, R w_node)
+// Parameters of feq of a cell's W.  In FP32 each is the sum of two numbers (_l: the second).
+// Rounded to one, the factor and the temperature put all of a cell's Maxwellian off alike, in
+// every step: R T was off by 2.3e-8 (root mean square, 40 x 40 x 100^2, 50 steps) where the general
+// kernels are by 0.8e-8.
+template <class R> struct Maxwell {
+    R amp, amp_l, u[2], u_l[2], beta, beta_l;
+};
+struct FF {                                    // h + l, |l| <= ulp(h) / 2
+    float h, l;
+};
+__device__ __forceinline__ FF ff_norm(float h, float l)
 {
-    // FP32: the moments rounded first, so that one thread does not hold its block for FP64
-    // divisions
-    const R rho = from_f64<R>(rho_d), ir = R(1) / rho, ux = from_f64<R>(mx) * ir, uy = from_f64<R>(my) * ir;
-    const R RT = from_f64<R>(rE) * ir - R(0.5) * (ux * ux + uy * uy), iRT = R(1) / RT;
-    par[0] = rho * iRT * R(0.5 / 3.14159265358979323846) * w_node;
-    par[1] = ux;
-    par[2] = uy;
-    par[3] = R(0.5) * iRT * (sizeof(R) == 4 ? R(1.4426950408889634) : R(1));
+    const float s = h + l;
+    return {s, l - (s - h)};
+}
+__device__ __forceinline__ FF ff_add(FF a, FF b)
+{
+    const float s = a.h + b.h, v = s - a.h;
+    return ff_norm(s, ((a.h - (s - v)) + (b.h - v)) + (a.l + b.l));
+}
+__device__ __forceinline__ FF ff_mul(FF a, FF b)
+{
+    const float p = a.h * b.h;
+    return ff_norm(p, fmaf(a.h, b.h, -p) + fmaf(a.h, b.l, a.l * b.h));
+}
+__device__ __forceinline__ FF ff_inv(FF a)
+{
+    const float q = recip<float>(a.h);
+    return ff_norm(q, q * (fmaf(-a.h, q, 1.0f) - a.l * q));
+}
+
+// w: W, and in FP32 what that leaves out of it.  (FP32: no FP64 divisions, for which the block would wait.)
+__device__ __forceinline__ void maxwell_of(Maxwell<float> &p, const float w[8], const DvmCartK<float> &K)
+{
+    constexpr double L = 0.5 * 1.4426950408889634;              // log2 e / 2
+    const FF r{w[0], w[4]}, ir = ff_inv(r), ux = ff_mul({w[1], w[5]}, ir), uy = ff_mul({w[2], w[6]}, ir);
+    const FF uu = ff_add(ff_mul(ux, ux), ff_mul(uy, uy));
+    const FF iRT = ff_inv(ff_add(ff_mul({w[3], w[7]}, ir), {-0.5f * uu.h, -0.5f * uu.l}));
+    const FF amp = ff_mul(ff_mul(r, iRT), {K.amp, K.amp_l}), beta = ff_mul(iRT, {(float)L, (float)(L - (double)(float)L)});
+    p = {amp.h, amp.l, {ux.h, uy.h}, {ux.l, uy.l}, beta.h, beta.l};
+}
+__device__ __forceinline__ void maxwell_of(Maxwell<double> &p, const double w[8], const DvmCartK<double> &K)
+{
+    const double ir = 1.0 / w[0], ux = w[1] * ir, uy = w[2] * ir, iRT = 1.0 / (w[3] * ir - 0.5 * (ux * ux + uy * uy));
+    p = {w[0] * iRT * K.amp, 0.0, {ux, uy}, {0.0, 0.0}, 0.5 * iRT, 0.0};
+}
+// By one warp, whose lanes 0 to 3 hold W in v.
+template <class R> __device__ __forceinline__ Maxwell<R> warp_maxwell(double v, const DvmCartK<R> &K)
+{
+    const R h = (R)v, l = sizeof(R) == 4 ? (R)(v - (double)h) : R(0);
+    R w[8];
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        w[k] = __shfl_sync(0xffffffffu, h, k);
+        w[4 + k] = __shfl_sync(0xffffffffu, l, k);
+    }
+    Maxwell<R> p;
+    maxwell_of(p, w, K);
+    return p;
 }
 // its one-axis factors (those along y with the density and node weight), by all threads of the block
-template <class R> __device__ __forceinline__ void cell_tables(const DvmCart &m, const R par[4], R *tab)
+template <class R> __device__ __forceinline__ void cell_tables(const DvmCart &m, const Maxwell<R> &p, R *tab)
 {
     const int nv = m.nv;
     for (int j = threadIdx.x; j < nv; j += blockDim.x) {
-        const R x = static_cast<const R *>(m.vnode)[j];
-        tab[j] = gauss<R>(x, par[1], par[3]);
-        tab[tab_row(nv, j)] = par[0] * gauss<R>(x, par[2], par[3]);
+        const R x = static_cast<const R *>(m.vnode)[j], gy = gauss<R>(x, p.u[1], p.beta, p.u_l[1], p.beta_l);
+        tab[j] = gauss<R>(x, p.u[0], p.beta, p.u_l[0], p.beta_l);
+        tab[tab_row(nv, j)] = fma(p.amp, gy, p.amp_l * gy);
     }
 }
 
@@ -191,10 +243,13 @@ template <class R>
 __global__ void __launch_bounds__(STATE_THREADS) k_dvc_init(const DvmCart m, const double *__restrict__ W, R *__restrict__ phi,
                                                            R *__restrict__ tab)
 {
-    __shared__ R par[4];
+    __shared__ Maxwell<R> par;
     const int64_t c = blockIdx.x;
     R *const t = tab + c * tab_size(m.nv);
-    if (threadIdx.x == 0) state_params<R>(par, W[4 * c], W[4 * c + 1], W[4 * c + 2], W[4 * c + 3], consts<R>(m).w_node);
+    if (threadIdx.x < 32) {
+        const Maxwell<R> p = warp_maxwell<R>(W[4 * c + (threadIdx.x & 3)], consts<R>(m));
+        if (threadIdx.x == 0) par = p;
+    }
     __syncthreads();
     cell_tables<R>(m, par, t);
     __syncthreads();
@@ -337,9 +392,9 @@ __global__ void __launch_bounds__(STATE_THREADS) k_dvc_states(const DvmCart m, c
     extern __shared__ __align__(16) unsigned char dyn[];
     const int nv = m.nv;
     R *const x = reinterpret_cast<R *>(dyn);
-    __shared__ double flux[4][4], wn[4];      // macroscopic fluxes, outward, less the reference's; W^{n+1}
+    __shared__ double flux[4][4];             // macroscopic fluxes, outward, less the reference's
     const DvmCartK<R> &K = consts<R>(m);
-    __shared__ R par[4];
+    __shared__ Maxwell<R> par;
     for (int j = threadIdx.x; j < nv; j += blockDim.x) x[j] = static_cast<const R *>(m.vnode)[j];
     step_dependency_wait();
     __syncthreads();
@@ -368,7 +423,7 @@ __global__ void __launch_bounds__(STATE_THREADS) k_dvc_states(const DvmCart m, c
             const R r = m0[mono(0, 0)] + d[0], e = R(0.5) * ((m0[mono(2, 0)] + d[ax == 0 ? 3 : 5]) + (m0[mono(0, 2)] + d[ax == 0 ? 5 : 3]));
             const R mx = m0[mono(1, 0)] + d[ax == 0 ? 1 : 2], my = m0[mono(0, 1)] + d[ax == 0 ? 2 : 1];
             const R ir = R(1) / r, ux = mx * ir, uy = my * ir, RT = e * ir - R(0.5) * (ux * ux + uy * uy), iRT = R(1) / RT;
-            const R pre = r * iRT * R(0.5 / 3.14159265358979323846) * K.w_node;
+            const R pre = r * iRT * K.amp;
             const R beta = R(0.5) * iRT * (sizeof(R) == 4 ? R(1.4426950408889634) : R(1));
             // tables, and their sums of powers 1..3 along (n) and 0..2 across (t), less the reference's (whose
             // odd ones are zero): the fluxes below are small differences
@@ -422,14 +477,14 @@ __global__ void __launch_bounds__(STATE_THREADS) k_dvc_states(const DvmCart m, c
         }
     }
     __syncthreads();
-    if (threadIdx.x < 4) {
-        const int k = threadIdx.x;
+    if (threadIdx.x < 32) {
+        const int k = lane & 3;
         const double w1 = W[4 * (int64_t)c + k] - m.kd.dtV * ((flux[0][k] + flux[1][k]) + (flux[2][k] + flux[3][k]));
-        W[4 * (int64_t)c + k] = w1;
-        wn[k] = w1;
+        __syncwarp();
+        if (lane < 4) W[4 * (int64_t)c + k] = w1;
+        const Maxwell<R> p = warp_maxwell<R>(w1, K);
+        if (lane == 0) par = p;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) state_params<R>(par, wn[0], wn[1], wn[2], wn[3], consts<R>(m).w_node);
     __syncthreads();
     cell_tables<R>(m, par, tab + (int64_t)c * tab_size(nv));
 }

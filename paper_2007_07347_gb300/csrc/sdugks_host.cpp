@@ -2363,15 +2363,16 @@ static void fill_dvm_cart(DvmCart &k, const sdugks_mesh &m, const CartGrid &g, c
     for (int j = 0; j < nv; j++) x[j] = rnd(node[j]);
     auto factors = [&](double *t, double ux, double uy) {
         for (int j = 0; j < nv; j++) {
-            t[j] = rnd(std::exp(-(node[j] - ux) * (node[j] - ux) / (2.0 * RT)));
-            t[nv + j] = rnd(h * h / (2.0 * pi * RT) * std::exp(-(node[j] - uy) * (node[j] - uy) / (2.0 * RT)));
+            // at the nodes as the gas has them: at others, the walls of a 33^2 grid drove R T up by 1e-10 a step
+            t[j] = rnd(std::exp(-(x[j] - ux) * (x[j] - ux) / (2.0 * RT)));
+            t[nv + j] = rnd(h * h / (2.0 * pi * RT) * std::exp(-(x[j] - uy) * (x[j] - uy) / (2.0 * RT)));
         }
     };
     m0.assign(2 * nv, 0.0);
     wt.assign(8 * nv, 0.0);
     factors(m0.data(), 0.0, 0.0);
     DvmCartK<double> &d = k.kd;
-    d.w_node = h * h;
+    d.amp = h * h / (2.0 * pi); d.amp_l = 0.0;
     d.a = (2.0 * tau - dt) / (2.0 * tau); d.b = dt / (2.0 * tau); d.c = 2.0 * tau / (2.0 * tau + dt);
     d.r = dt / tau; d.inv1r = 1.0 / (1.0 + dt / tau); d.dtV = dt / (g.dx * g.dy);
     d.len[0] = g.dy; d.len[1] = g.dx;
@@ -2432,7 +2433,7 @@ static void fill_dvm_cart(DvmCart &k, const sdugks_mesh &m, const CartGrid &g, c
         }
     }
     DvmCartK<float> &f = k.kf;
-    f.w_node = (float)d.w_node; f.a = (float)d.a; f.b = (float)d.b; f.c = (float)d.c; f.r = (float)d.r;
+    f.amp = (float)d.amp; f.amp_l = (float)(d.amp - (double)f.amp); f.a = (float)d.a; f.b = (float)d.b; f.c = (float)d.c; f.r = (float)d.r;
     f.inv1r = (float)d.inv1r; f.dtV = (float)d.dtV;
     for (int q = 0; q < 2; q++) { f.len[q] = (float)d.len[q]; f.kh[q] = (float)d.kh[q]; f.kdt[q] = (float)d.kdt[q]; }
     for (int q = 0; q < 15; q++) f.m0f[q] = (float)d.m0f[q];

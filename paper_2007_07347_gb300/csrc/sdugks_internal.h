@@ -299,7 +299,8 @@ struct DvmWall {
                                // less the reference's, for a cell that holds the reference
 };
 template <class R> struct DvmCartK {
-    R w_node, a, b, c, r, inv1r, dtV;
+    R amp, amp_l;              // node weight / (2 pi); what amp leaves out
+    R a, b, c, r, inv1r, dtV;
     R len[2];                  // length of a face of constant x, y
     R kh[2], kdt[2];           // h / 2 and dt along x and y, times 1 / (2 h)
     R m0f[15], m0s[2][2];      // moments of the reference; of its factors along x and y (powers 0 and 2)

@@ -86,3 +86,25 @@ def test_fp64_error_does_not_grow(n, nv, kn, steps):
         device_bytes = d.sizes()["device_bytes"]
     assert device_bytes > 1.5 * N * nv * nv * 16        # the second is the general path, with its face fluxes
     assert np.sqrt(np.sum((v[0] - v[1]) ** 2) / np.sum(v[1] ** 2)) <= 2e-14
+
+
+@pytest.mark.parametrize("n,nv,kn,steps,bound", [(40, 100, 1.0, 50, 1.2e-8), (40, 33, 8.0, 100, 2e-8)])
+def test_fp32_temperature_noise(n, nv, kn, steps, bound):
+    """R T in FP32 against FP64, root mean square.  The general kernels, whose rounding errors
+    average over nv^2 nodes, are 0.8e-8 and 1.45e-8 off; a rounding that all nodes of a cell share
+    (their Maxwellian's temperature or factor) gave 2.3e-8 and 2.7e-8 plus a drift of 2e-8.  About
+    half way between."""
+    S = _S()
+    c = M.micro_cavity(n, kn, nv=nv)
+    rng = np.random.default_rng(3)
+    N = n * n
+    x = (np.arange(n) + 0.5) / n
+    s = np.outer(np.sin(np.pi * x), np.sin(np.pi * x)).ravel()
+    rho, RT = 1 + 0.01 * s, 0.5 + 0.01 * s
+    u = 0.05 * s[:, None] * rng.normal(size=2)
+    T = []
+    for prec in ("fp64", "fp32"):
+        d = S.Dvm.from_case(c, prec).init(rho, u, RT)
+        d.step(steps)
+        T.append(d.macros()[2])
+    assert np.sqrt(np.mean((T[1] - T[0]) ** 2)) <= bound
