@@ -13,6 +13,22 @@ def _S():
     return S
 
 
+@pytest.mark.parametrize("n,tau", [(20, 9.5175), (20, 9.8375), (240, 9.6925)])
+def test_fp64_gas_at_rest_keeps_f(n, tau):
+    """rho = 1.12 at rest, dt = 0.25, 600 steps, tau such that the two fractions rounded by
+    themselves miss their whole by more than an ulp.  W does not change.  f^{n+1} = inv f + ri feq is
+    f itself, after rounding, wherever f is feq to half an ulp; the initial f and ri feq / ri may be one
+    ulp apart.  Within two ulp, where fractions rounded by themselves gave 37."""
+    S = _S()
+    s = S.Solver.from_case(M.periodic_box(n, n, tau=tau, dt=0.25), "fp64").init(np.full(n * n, 1.12), None)
+    f0, W0 = s.get_state()
+    s.step(600)
+    f, W = s.get_state()
+    np.testing.assert_array_equal(W, W0)
+    w = np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)
+    assert (np.abs(f - f0) / np.spacing(1.12 * w)).max() <= 2
+
+
 def test_strips_are_no_further_off_than_blocks():
     """FP32 448^2 against FP64, 300 steps: the marching form and the block form (which tensor-copy
     staging runs) hold the same equations in other sums; 2-norm of u, 5 % for the other rounding."""
