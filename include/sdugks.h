@@ -316,12 +316,14 @@ void sdugks_autotune_clear(void);
 /* ---- batched solves ----------------------------------------------------------- */
 /* Many independent uniform-grid solves (cavities, channels) of different sizes and
  * Reynolds numbers advanced together; steps replay a captured CUDA graph.  In FP32 a
- * step is one launch per 96 instances over their (instance, strip, range of rows) items,
- * one marching warp each.  Instances with a symmetry side or an odd width between
- * periodic sides, and the 16-bit storages, are stepped by one launch over the (instance,
- * 16x8 block) work list, one CTA per item (or, if the autotuner prefers it, a fixed grid
- * of CTAs walking the list).  An instance's arithmetic depends on its own grid only, so
- * its results do not depend on what else is in the batch.  Instances
+ * step of a batch that fills the device for many waves is one launch per 96 instances
+ * over their (instance, strip, range of rows) items, one marching warp each; of a smaller
+ * one, one launch over its (instance, 16x8 block) items, with the same results to the last bit.
+ * Instances with a symmetry side or an odd width between periodic sides, and the 16-bit
+ * storages, are stepped by one launch of another kernel over their blocks, one CTA per item (or, if
+ * the autotuner prefers it, a fixed grid of CTAs walking the list).  An instance's
+ * arithmetic depends on its own grid only, so its results do not depend on what else is in
+ * the batch.  Instances
  * are admitted while the batch's device pool has room for their state (admission
  * by device-memory footprint) and can be removed at any step boundary, which frees
  * their memory for new ones (continuous batching). */
@@ -340,6 +342,7 @@ typedef struct sdugks_batch_status {
     int32_t precision;
     int32_t per_item;        /* 1: one CTA per work item; 0: a fixed grid walks the
                                 work list                                           */
+    int32_t march;           /* 1: FP32 instances step by marching warps, 0: by blocks  */
 } sdugks_batch_status;
 
 /* Create a batch with a device pool of pool_bytes and room for max_instances

@@ -36,7 +36,8 @@ CU_UNITS = {
     "k_dvm_cart.cu": [],
 }
 CXX_UNITS = ["sdugks_host.cpp"]
-HEADERS = ["sdugks_internal.h", "d2q9.cuh", "step_tiled.cuh", "step_cart.cuh", "step_strip.cuh"]
+HEADERS = ["sdugks_internal.h", "d2q9.cuh", "step_tiled.cuh", "step_cart.cuh", "step_strip.cuh",
+           "step_strip_block.cuh"]
 
 
 def _sources():

@@ -1,5 +1,6 @@
-// k_strip.cu -- the marching-warp Cartesian step (FP32) of single solves and of batches.
-#include "step_strip.cuh"
+// k_strip.cu -- the marching-warp Cartesian step (FP32) of single solves and of batches, and
+// its form by blocks for small batches.
+#include "step_strip_block.cuh"
 
 namespace sdugks {
 
@@ -23,6 +24,25 @@ k_strip_batch(const __grid_constant__ StripGroup G, const int2 *__restrict__ ite
     step_dependency_wait();
     const int q = __shfl_sync(0xffffffffu, it.x, 0), y = __shfl_sync(0xffffffffu, it.y, 0);
     strip_item(G.inst[q], par, y & 0xFFFF, y >> 16, rows, smem_raw);
+}
+
+// Batched, by blocks (step_strip_block.cuh): one CTA per (instance, block x | block y << 16)
+// item.  The items and the records are written by the host only and are read before the wait.
+template <bool WIDE>
+__global__ void __launch_bounds__(sb_threads<WIDE>(), sb_ctas<WIDE>())
+k_strip_block_batch(const StripInst *__restrict__ insts, const int2 *__restrict__ items, int par)
+{
+    __shared__ __align__(16) StripBlockSmem S;
+    const int2 it = items[blockIdx.x];
+    static_assert(sizeof(StripInst) % 8 == 0 && sizeof(StripInst) / 8 <= sb_threads<WIDE>(), "the record in one round");
+    if (threadIdx.x < sizeof(StripInst) / 8)
+        reinterpret_cast<uint64_t *>(&S.m)[threadIdx.x] = reinterpret_cast<const uint64_t *>(insts + it.x)[threadIdx.x];
+    step_dependency_wait();
+    __syncthreads();
+    const int x0 = (it.y & 0xFFFF) * 16, y0 = (it.y >> 16) * BATCH_TY;
+    const bool inside = x0 >= 2 && x0 + 18 <= S.m.nx && y0 >= 2 && y0 + BATCH_TY + 2 <= S.m.ny;
+    if (inside) strip_block<false, WIDE>(S, par, x0, y0);
+    else strip_block<true, WIDE>(S, par, x0, y0);
 }
 
 bool strip_fits(const CartInst &m, int prec)
@@ -77,8 +97,8 @@ void fill_strip(const CartInst &m, StripInst &s)
         s.g[x] = two(whole_less(bg, lv)); s.bg[x] = two(part_of(bg, lv));
     }
     const double ax = 0.5 * m.ihx, ay = 0.5 * m.ihy;
-    signs(s.xdt, m.dt * ax); signs(s.xh, 0.25); signs(s.xo, 0.25 - m.dt * ax);
-    signs(s.ydt, m.dt * ay); signs(s.yh, 0.25); signs(s.yo, 0.25 - m.dt * ay);
+    signs(s.xdt, m.dt * ax); signs(s.xh, STRIP_XH); signs(s.xo, 0.25 - m.dt * ax);
+    signs(s.ydt, m.dt * ay); signs(s.yh, STRIP_XH); signs(s.yo, 0.25 - m.dt * ay);
 }
 
 cudaError_t prepare_strip()
@@ -95,6 +115,23 @@ cudaError_t launch_strip_batch(const StripGroup &g, const int2 *items, int n_ite
                                int parity, cudaStream_t st)
 {
     return launch_step_kernel(early, k_strip_batch, dim3(n_items), dim3(32), STRIP_SMEM, st, g, items, parity, rows);
+}
+
+cudaError_t launch_strip_blocks(const StripInst *insts, const int2 *items, int n_items, bool wide, bool early, int parity,
+                                cudaStream_t st)
+{
+    if (wide)
+        return launch_step_kernel(early, k_strip_block_batch<true>, dim3(n_items), dim3(sb_threads<true>()), 0, st, insts, items, parity);
+    return launch_step_kernel(early, k_strip_block_batch<false>, dim3(n_items), dim3(sb_threads<false>()), 0, st, insts, items, parity);
+}
+
+int strip_block_slots(bool wide)
+{
+    int dev = 0, n_sm = 1, n = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    const cudaError_t e = wide ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_strip_block_batch<true>, sb_threads<true>(), 0)
+                               : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_strip_block_batch<false>, sb_threads<false>(), 0);
+    return n_sm * (e != cudaSuccess || n < 1 ? 1 : n);
 }
 
 cudaError_t launch_step_strip(const StripInst &s, int rows, bool early, int parity, cudaStream_t st)

@@ -1860,7 +1860,7 @@ struct BatchInst {
     size_t off, bytes;
     int64_t admitted_at;            // batch step at admission
     int64_t ntiles;
-    bool strip;                     // steps by marching warps (else by blocks)
+    bool strip;                     // steps by marching warps or their block form (else by cart_tile's blocks)
     std::vector<int64_t> lattice;   // caller's cell c -> lattice position i + nx j
 };
 
@@ -1889,13 +1889,15 @@ struct sdugks_batch {
     // device tables (fixed addresses, sized for max_inst and max_items)
     CartInst *d_inst = nullptr;
     int2 *d_items = nullptr;
-    int *d_nitems = nullptr;            // [2]: work items, and those of the instances stepped by blocks (listed first)
+    int *d_nitems = nullptr;            // [2]: work items, and those of the instances stepped by cart_tile's blocks (listed first)
+    int64_t n_block = 0;                // the latter
+    // instances stepped by marching warps, or by their block form (the items past n_block)
+    bool march = false;
+    StripInst *d_strip = nullptr;       // records of the block form, by instance
     int2 *d_sitems = nullptr;           // items of the marching warps, by group
-    struct Group { StripGroup g; int64_t first, n; };
+    struct Group { StripGroup g; int64_t first, n; int rows; bool early; };
     std::vector<Group> groups;
-    int strip_rows = 0;
-    bool strip_early = true;
-    int64_t n_block = 0;                // items stepped by blocks
+    bool strip_early = true;            // of the block form's launches
     double *d_partial = nullptr, *d_out = nullptr;
     double *h_out = nullptr;            // pinned [max_inst][4]
     double *d_stage = nullptr;          // [max_cells_one][3] staging for add/get
@@ -1905,8 +1907,10 @@ struct sdugks_batch {
     bool per_item = true;                       // one CTA per work item (the grid follows the list)
     int graph_steps = 64;
     cudaGraphExec_t graph = nullptr;
-    bool graph_strips = false;                  // the graph holds launches of marching warps
-    int64_t n_strip_slots = 1;
+    bool graph_march = false;                   // the graph holds launches of marching warps
+    int64_t graph_items = -1, graph_block = -1; // the item counts that its grids were sized for
+    bool graph_early = false;
+    int64_t n_strip_slots = 1, n_strip_block_slots = 1, n_strip_wide_slots = 1;
 };
 
 // CTAs of a block step launch: one per block item (at least one), or the walking form's grid
@@ -1915,21 +1919,29 @@ static int batch_launch_grid(const sdugks_batch *b)
     return b->per_item ? (int)(b->n_block > 0 ? b->n_block : 1) : b->grid;
 }
 
-// One step of every instance: the marching warps of each group, then the blocks (the
-// instances are independent; each launch waits for the one before it).
+// One step of every instance: the marching warps of each group or their block form, then
+// cart_tile's blocks (the instances are independent; each launch waits for the one before it).
 static cudaError_t batch_launch_step(const sdugks_batch *b, int parity, bool per_item, int grid, cudaStream_t st)
 {
     cudaError_t e = cudaSuccess;
+    const bool single = st != b->cap_stream;          // not into a graph: see early_start
+    const int64_t n_strip = b->n_items - b->n_block;
     for (const auto &g : b->groups)
         if (e == cudaSuccess)
-            e = launch_strip_batch(g.g, b->d_sitems + g.first, (int)g.n, b->strip_rows, b->strip_early || st != b->cap_stream, parity, st);
-    if (e == cudaSuccess && (b->n_block > 0 || b->groups.empty()))
+            e = launch_strip_batch(g.g, b->d_sitems + g.first, (int)g.n, g.rows, g.early || single, parity, st);
+    if (!b->march && n_strip > 0)
+        e = launch_strip_blocks(b->d_strip, b->d_items + b->n_block, (int)n_strip, n_strip <= b->n_strip_wide_slots,
+                                b->strip_early || single, parity, st);
+    if (e == cudaSuccess && (b->n_block > 0 || n_strip == 0))
         e = launch_step_batch(b->prec, b->d_inst, b->d_items, b->d_nitems + 1, grid, per_item, parity, st);
     return e;
 }
 
 static int batch_upload_tables(sdugks_batch *b)
 {
+    int64_t total = 0;
+    for (const auto &i : b->inst) total += i.ntiles;
+    if (total > b->max_items) return fail(SDUGKS_ERR_FULL, "batch work list full");      // before anything changes
     std::vector<CartInst> h(b->inst.size());
     std::vector<int2> items, sitems;
     // instances stepped by blocks first: their items are the head of the list
@@ -1947,47 +1959,81 @@ static int batch_upload_tables(sdugks_batch *b)
         }
         if (!strip) b->n_block = (int64_t)items.size();
     }
-    if ((int64_t)items.size() > b->max_items) return fail(SDUGKS_ERR_FULL, "batch work list full");
     b->n_items = (int64_t)items.size();
-    // the marching warps' items, in groups of instances
-    std::vector<const CartInst *> si;
-    int max_ny = 1;
-    for (const auto &i : b->inst)
-        if (i.strip) { si.push_back(&i.ci); max_ny = std::max(max_ny, i.ci.ny); }
-    b->groups.clear();
-    if (!si.empty()) {
-        auto count = [&](int rows) {
-            int64_t n = 0;
-            for (const CartInst *c : si) n += (int64_t)strip_count(c->nx, c->periodic_x != 0) * ((c->ny + rows - 1) / rows);
-            return n > b->max_items ? INT64_MAX / 4096 : n;      // past the list's room
-        };
-        double cost;
-        b->strip_rows = strip_rows(b->n_strip_slots, max_ny, count, cost);
-        for (size_t q = 0; q < si.size(); q++) {
-            if (q % STRIP_GROUP == 0) {
-                b->groups.emplace_back();
-                std::memset(&b->groups.back(), 0, sizeof(b->groups.back()));
-                b->groups.back().first = (int64_t)sitems.size();
-            }
-            auto &G = b->groups.back();
-            const int k = (int)(q % STRIP_GROUP), strips = strip_count(si[q]->nx, si[q]->periodic_x != 0);
-            fill_strip(*si[q], G.g.inst[k]);
-            const int segs = (si[q]->ny + b->strip_rows - 1) / b->strip_rows;
-            for (int t = 0; t < segs; t++)
-                for (int x = 0; x < strips; x++) sitems.push_back(make_int2(k, x | (t << 16)));
-            G.n = (int64_t)sitems.size() - G.first;
+    // FP32 instances without a symmetry side or an odd wrap: marching warps, or their block form where
+    // the whole list is too little work for those.  Measured (GB300, us per step of n x n cavities, marching /
+    // blocks): 1 of 32^2 4.4 / 2.7, 4 of 128^2 9.1 / 5.0, 1 of 256^2 8.3 / 5.0, 64 of 32^2 10.0 / 5.2, 32 of 64^2
+    // 8.1 / 8.3, 4 of 256^2 14.2 / 13.7, 1 of 512^2 11.9 / 13.5, 64 of 64^2 12.5 / 14.6, 8 of 256^2 22.6 / 25.3,
+    // 2 of 512^2 19.2 / 24.9.  A unit of strip_rows' cost takes 1.9 to 2.3 us, the more the narrower the grids (edge
+    // strips), blocks 1.9 us and 5.8 ns each.
+    std::vector<size_t> si;
+    std::vector<StripInst> records;
+    for (size_t q = 0; q < b->inst.size(); q++)
+        if (b->inst[q].strip) si.push_back(q);
+    const int64_t blocks = b->n_items - b->n_block;
+    // groups of instances (one launch each, one after the other), as equal as can be
+    const size_t ng = (si.size() + STRIP_GROUP - 1) / STRIP_GROUP;
+    std::vector<int> rows(ng);
+    double cost = 0.0;
+    for (size_t g = 0; g < ng; g++) {
+        const size_t lo = si.size() * g / ng, hi = si.size() * (g + 1) / ng;
+        int max_ny = 1;
+        int64_t room = (b->max_items - b->n_items) / (int64_t)ng;        // in the list of the marching warps' items
+        for (size_t q = lo; q < hi; q++) {
+            max_ny = std::max(max_ny, b->inst[si[q]].ci.ny);
+            room += b->inst[si[q]].ntiles;
         }
-        b->strip_early = early_start((int64_t)sitems.size(), b->n_strip_slots, b->n_sm);
+        auto count = [&](int r) {
+            int64_t n = 0;
+            for (size_t q = lo; q < hi; q++) {
+                const CartInst &c = b->inst[si[q]].ci;
+                n += (int64_t)strip_count(c.nx, c.periodic_x != 0) * ((c.ny + r - 1) / r);
+            }
+            return n > room ? INT64_MAX / 4096 : n;      // eight rows, or all of fewer, fit always
+        };
+        double c;
+        rows[g] = strip_rows(b->n_strip_slots, max_ny, count, c);
+        cost += c;
+    }
+    b->groups.clear();
+    b->march = ng > 0 && 2.1 * cost < 1.9 + 5.8e-3 * (double)blocks;
+    b->strip_early = early_start(blocks, b->n_strip_block_slots, b->n_sm);
+    if (b->march) {
+        b->groups.resize(ng);
+        std::memset(b->groups.data(), 0, ng * sizeof b->groups[0]);
+        for (size_t g = 0; g < ng; g++) {
+            auto &G = b->groups[g];
+            const size_t lo = si.size() * g / ng, hi = si.size() * (g + 1) / ng;
+            G.first = (int64_t)sitems.size();
+            G.rows = rows[g];
+            for (size_t q = lo; q < hi; q++) {
+                const CartInst &c = b->inst[si[q]].ci;
+                fill_strip(c, G.g.inst[q - lo]);
+                const int segs = (c.ny + G.rows - 1) / G.rows, strips = strip_count(c.nx, c.periodic_x != 0);
+                for (int t = 0; t < segs; t++)
+                    for (int x = 0; x < strips; x++) sitems.push_back(make_int2((int)(q - lo), x | (t << 16)));
+            }
+            G.n = (int64_t)sitems.size() - G.first;
+            G.early = early_start(G.n, b->n_strip_slots, b->n_sm);
+        }
+    } else if (ng > 0) {
+        records.resize(b->inst.size());
+        for (const size_t q : si) fill_strip(b->inst[q].ci, records[q]);
     }
     const int ni[2] = {(int)b->n_items, (int)b->n_block};
     if (!h.empty()) CUDA_TRY(cudaMemcpyAsync(b->d_inst, h.data(), h.size() * sizeof(CartInst), cudaMemcpyHostToDevice, b->stream));
     if (!items.empty()) CUDA_TRY(cudaMemcpyAsync(b->d_items, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice, b->stream));
     if (!sitems.empty()) CUDA_TRY(cudaMemcpyAsync(b->d_sitems, sitems.data(), sitems.size() * sizeof(int2), cudaMemcpyHostToDevice, b->stream));
+    if (!records.empty()) CUDA_TRY(cudaMemcpyAsync(b->d_strip, records.data(), records.size() * sizeof(StripInst), cudaMemcpyHostToDevice, b->stream));
     CUDA_TRY(cudaMemcpyAsync(b->d_nitems, ni, sizeof ni, cudaMemcpyHostToDevice, b->stream));
     CUDA_TRY(cudaStreamSynchronize(b->stream));   // the host vectors go out of scope
-    // a graph's launches carry the old list: grids of its item counts, records of its
-    // instances (destroyed after the synchronisation, so no launch of it is still running)
-    if (b->graph && (b->per_item || !b->groups.empty() || b->graph_strips)) {
+    // a graph's launches carry the old list: marching warps the records of its instances, the
+    // others grids of its item counts (the walking form has a fixed one).  Destroyed after the
+    // synchronisation, so no launch of it is still running
+    const int64_t n_strip = blocks;
+    const bool same = n_strip == b->graph_items - b->graph_block && b->strip_early == b->graph_early &&
+                      (b->per_item || n_strip > 0 ? b->n_block == b->graph_block : (b->n_block > 0) == (b->graph_block > 0));
+    if (b->graph && (b->march || b->graph_march || !same)) {
         cudaGraphExecDestroy(b->graph);
         b->graph = nullptr;
     }
@@ -2017,6 +2063,7 @@ extern "C" int sdugks_batch_create(int64_t pool_bytes, int32_t precision, int32_
     if (e == cudaSuccess) e = cudaMalloc(&b->d_inst, sizeof(CartInst) * (size_t)max_instances);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_items, sizeof(int2) * (size_t)b->max_items);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_sitems, sizeof(int2) * (size_t)(precision == SDUGKS_FP32 ? b->max_items : 1));
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_strip, sizeof(StripInst) * (size_t)(precision == SDUGKS_FP32 ? max_instances : 1));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_nitems, 2 * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_partial, sizeof(double) * 4 * (size_t)b->max_items);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_out, sizeof(double) * 4 * (size_t)max_instances);
@@ -2032,6 +2079,8 @@ extern "C" int sdugks_batch_create(int64_t pool_bytes, int32_t precision, int32_
     b->ctas_per_sm = batch_ctas_per_sm(precision);
     b->grid = b->n_sm * b->ctas_per_sm;
     b->n_strip_slots = strip_slots();
+    b->n_strip_block_slots = strip_block_slots(false);
+    b->n_strip_wide_slots = strip_block_slots(true);
     *out = b;
     return SDUGKS_OK;
 }
@@ -2152,7 +2201,9 @@ static int batch_ensure_graph(sdugks_batch *b)
     e = cudaGraphInstantiate(&b->graph, g, 0);
     cudaGraphDestroy(g);
     CUDA_TRY(e);
-    b->graph_strips = !b->groups.empty();
+    b->graph_march = b->march;
+    b->graph_items = b->n_items; b->graph_block = b->n_block;
+    b->graph_early = b->strip_early;
     return SDUGKS_OK;
 }
 
@@ -2283,6 +2334,7 @@ extern "C" int sdugks_batch_info(const sdugks_batch *b, sdugks_batch_status *o)
     o->graph_steps = b->graph_steps;
     o->precision = b->prec;
     o->per_item = b->per_item ? 1 : 0;
+    o->march = b->march ? 1 : 0;
     return SDUGKS_OK;
 }
 
@@ -2297,6 +2349,7 @@ extern "C" void sdugks_batch_destroy(sdugks_batch *b)
     cudaFree(b->d_inst);
     cudaFree(b->d_items);
     cudaFree(b->d_sitems);
+    cudaFree(b->d_strip);
     cudaFree(b->d_nitems);
     cudaFree(b->d_partial);
     cudaFree(b->d_out);

@@ -201,6 +201,11 @@ static_assert(sizeof(StripGroup) <= 32000, "a group is a kernel parameter");
 cudaError_t prepare_strip_batch();
 cudaError_t launch_strip_batch(const StripGroup &g, const int2 *items, int n_items, int rows, bool early, int parity,
                                cudaStream_t st);
+// by blocks of 16 x BATCH_TY cells, one CTA per (instance, block) item, the records in device
+// memory: the same bits as the marching warps.  wide: for lists within strip_block_slots(true)
+cudaError_t launch_strip_blocks(const StripInst *insts, const int2 *items, int n_items, bool wide, bool early, int parity,
+                                cudaStream_t st);
+int strip_block_slots(bool wide);                            // resident CTAs of the device
 // batched: every (instance, tile) item of the list, one per CTA (per_item: grid >= the
 // item count) or grid-stride over a fixed grid
 cudaError_t prepare_batch(int prec);

@@ -35,6 +35,7 @@ constexpr int STRIP_W = 64;        // columns a warp stages (two per lane)
 constexpr int STRIP_STEP = 60;     // columns from one strip to the next
 constexpr int STRIP_RING = 4;      // rows of f^n, W^n in shared memory: j - 1 .. j + 2
 constexpr int STRIP_CTAS = 8;      // warps (one-warp CTAs) per SM
+constexpr float STRIP_XH = 0.25f;  // (h / 2) / (2 h): StripInst's xh and yh
 
 // Shared memory of a row: W^n (3 planes of 32 x two cells), then f^n (9 planes).
 constexpr int STRIP_WB = 3 * 32 * 16, STRIP_ROW = STRIP_WB + NQ * 32 * 8;
@@ -133,6 +134,60 @@ __device__ __forceinline__ void strip_store(float *p, int n, const float2 v[NQ],
 #undef SDUGKS_ST
 }
 
+// Two cells' values of every plane at p, of the cells that are `on`; ODD: where one of the
+// two alone can be.
+template <class T, int N, class P>
+__device__ __forceinline__ void strip_put_n(P *p, int np, const T v[N], bool on0, bool on1, bool odd)
+{
+    strip_store(p, np, v, on0 && on1);
+    if (odd && on0 != on1) {
+#pragma unroll
+        for (int k = 0; k < N; k++) p[(int64_t)np * k + (on0 ? 0 : 1)] = on0 ? v[k].x : v[k].y;
+    }
+}
+__device__ __forceinline__ void strip_put(double *p, int np, const double2 v[3], bool on0, bool on1, bool odd)
+{
+    strip_put_n<double2, 3>(p, np, v, on0, on1, odd);
+}
+__device__ __forceinline__ void strip_put(float *p, int np, const float2 v[NQ], bool on0, bool on1, bool odd)
+{
+    strip_put_n<float2, NQ>(p, np, v, on0, on1, odd);
+}
+
+// W^{n+1} and f^{n+1} of two cells from their flux sums F; W^n and f^n by W(k), f(a), the
+// results to put_W and put_f.
+template <class GetW, class GetF, class PutW, class PutF>
+__device__ __forceinline__ void strip_update(const float2 F[NQ], const StripInst &m, GetW &&W, GetF &&f, PutW &&put_W,
+                                             PutF &&put_f)
+{
+    const float2 sm1 = __fadd2_rn(__fadd2_rn(F[1], F[3]), __fadd2_rn(F[5], F[7]));
+    const float2 sm2 = __fadd2_rn(__fadd2_rn(F[2], F[4]), __fadd2_rn(F[6], F[8]));
+    const float2 d57 = sub2(F[5], F[7]), d68 = sub2(F[6], F[8]);
+    float2 d[3] = {__fadd2_rn(sm1, sm2), __fadd2_rn(sub2(F[1], F[3]), sub2(d57, d68)),
+                   __fadd2_rn(sub2(F[2], F[4]), __fadd2_rn(d57, d68))};
+    float2 b0, m1, m2;
+    {
+        double2 w[3], dd[3];
+        f2d_six(d, dd);
+#pragma unroll
+        for (int k = 0; k < 3; k++) w[k] = W(k);
+        b0 = d2f2(w[0]); m1 = d2f2(w[1]); m2 = d2f2(w[2]);
+#pragma unroll
+        for (int k = 0; k < 3; k++) w[k] = make_double2(w[k].x - dd[k].x, w[k].y - dd[k].y);
+        put_W(w);
+    }
+    const float2 drho1 = sub2(b0, d[0]), rho1 = __fadd2_rn(dup(1.0f), drho1), inv = rcp2(rho1);
+    const float2 ux1 = __fmul2_rn(sub2(m1, d[1]), inv), uy1 = __fmul2_rn(sub2(m2, d[2]), inv);
+    float2 fe[NQ], v[NQ];
+    feq_pair(__fmul2_rn(m.ri, drho1), __fmul2_rn(m.ri, rho1), ux1, uy1, fe);
+#pragma unroll
+    for (int a = 0; a < NQ; a++) {
+        const float2 fn = f(a);
+        v[a] = __ffma2_rn(m.inv, a == 0 ? fn : sub2(fn, F[a]), fe[a]);
+    }
+    put_f(v);
+}
+
 // Interface moments of the pair of faces, then their six fluxes times dt / V, from the
 // six crossing distributions v[6] (slot order XSLOT_A / YSLOT_A) and the sums of the three
 // tangential ones over both sides: AX 0: (0, 2, 4), AX 1: (0, 1, 3).  The fluxes carry no
@@ -191,6 +246,20 @@ __device__ __forceinline__ void strip_boundary(float2 F[NQ], const float2 out[3]
     }
 }
 
+// rho - 1, rho and u of two cells from W^n
+__device__ __forceinline__ void strip_state(double2 w0, double2 w1, double2 w2, float2 &b0, float2 &rho, float2 &ux, float2 &uy)
+{
+    b0 = d2f2(w0);
+    rho = __fadd2_rn(dup(1.0f), b0);
+    const float2 inv = rcp2(rho);
+    ux = __fmul2_rn(d2f2(w1), inv);
+    uy = __fmul2_rn(d2f2(w2), inv);
+}
+
+// F plus or minus the unsigned flux of a velocity with the sign sg.
+__device__ __forceinline__ float2 strip_minus(float2 F, float2 fl, int sg) { return sg > 0 ? sub2(F, fl) : __fadd2_rn(F, fl); }
+__device__ __forceinline__ float2 strip_plus(float2 F, float2 fl, int sg) { return sg > 0 ? __fadd2_rn(F, fl) : sub2(F, fl); }
+
 // One warp: rows [y0, y1) of the strip whose first staged column is xb; reads buffer
 // `par`, writes buffer 1 - par.  sm: the warp's shared memory.  EDGE: the strip meets
 // a grid side in x (a wall or a wrap) or ends past the grid; other strips update lanes
@@ -234,11 +303,7 @@ __device__ __forceinline__ void strip_march(const StripInst &m, int par, int xb,
     auto row_f = [&](int slot, int a) { return *reinterpret_cast<const float2 *>(lf + slot * STRIP_ROW + a * 256); };
     // rho - 1, rho and u of a row that has arrived
     auto state = [&](int slot, float2 &b0, float2 &rho, float2 &ux, float2 &uy) {
-        b0 = d2f2(row_W(slot, 0));
-        rho = __fadd2_rn(dup(1.0f), b0);
-        const float2 inv = rcp2(rho);
-        ux = __fmul2_rn(d2f2(row_W(slot, 1)), inv);
-        uy = __fmul2_rn(d2f2(row_W(slot, 2)), inv);
+        strip_state(row_W(slot, 0), row_W(slot, 1), row_W(slot, 2), b0, rho, ux, uy);
     };
     // fbar+ of a row that has arrived
     auto stage = [&](int slot, float2 out[NQ]) {
@@ -256,45 +321,10 @@ __device__ __forceinline__ void strip_march(const StripInst &m, int par, int xb,
 
     // W^{n+1} and f^{n+1} of the row in `slot` (at row `row` of the grid) from its flux sums
     auto update = [&](int slot, int row, const float2 F[NQ]) {
-        const float2 sm1 = __fadd2_rn(__fadd2_rn(F[1], F[3]), __fadd2_rn(F[5], F[7]));
-        const float2 sm2 = __fadd2_rn(__fadd2_rn(F[2], F[4]), __fadd2_rn(F[6], F[8]));
-        const float2 d57 = sub2(F[5], F[7]), d68 = sub2(F[6], F[8]);
-        float2 d[3] = {__fadd2_rn(sm1, sm2), __fadd2_rn(sub2(F[1], F[3]), sub2(d57, d68)),
-                       __fadd2_rn(sub2(F[2], F[4]), __fadd2_rn(d57, d68))};
         const int64_t o = (int64_t)pitch * row;
-        float2 b0, m1, m2;
-        {
-            double2 w[3], dd[3];
-            f2d_six(d, dd);
-#pragma unroll
-            for (int k = 0; k < 3; k++) w[k] = row_W(slot, k);
-            b0 = d2f2(w[0]); m1 = d2f2(w[1]); m2 = d2f2(w[2]);
-#pragma unroll
-            for (int k = 0; k < 3; k++) {
-                w[k] = make_double2(w[k].x - dd[k].x, w[k].y - dd[k].y);
-            }
-            double *const p = Wout + o;
-            strip_store(p, np, w, up0 && up1);
-            if (EDGE && up0 != up1) {
-#pragma unroll
-                for (int k = 0; k < 3; k++) p[(int64_t)np * k + (up0 ? 0 : 1)] = up0 ? w[k].x : w[k].y;
-            }
-        }
-        const float2 drho1 = sub2(b0, d[0]), rho1 = __fadd2_rn(dup(1.0f), drho1), inv = rcp2(rho1);
-        const float2 ux1 = __fmul2_rn(sub2(m1, d[1]), inv), uy1 = __fmul2_rn(sub2(m2, d[2]), inv);
-        float2 fe[NQ], v[NQ];
-        feq_pair(__fmul2_rn(m.ri, drho1), __fmul2_rn(m.ri, rho1), ux1, uy1, fe);
-#pragma unroll
-        for (int a = 0; a < NQ; a++) {
-            const float2 fn = row_f(slot, a);
-            v[a] = __ffma2_rn(m.inv, a == 0 ? fn : sub2(fn, F[a]), fe[a]);
-        }
-        float *const p = fout + o;
-        strip_store(p, np, v, up0 && up1);
-        if (EDGE && up0 != up1) {
-#pragma unroll
-            for (int a = 0; a < NQ; a++) p[(int64_t)np * a + (up0 ? 0 : 1)] = up0 ? v[a].x : v[a].y;
-        }
+        strip_update(F, m, [&](int k) { return row_W(slot, k); }, [&](int a) { return row_f(slot, a); },
+                     [&](const double2 w[3]) { strip_put(Wout + o, np, w, up0, up1, EDGE); },
+                     [&](const float2 v[NQ]) { strip_put(fout + o, np, v, up0, up1, EDGE); });
     };
     // a boundary face of the row in `slot` in direction D
     auto boundary = [&](auto dir, int slot, int side, float2 F[NQ], const float2 out[3], bool on0, bool on1) {
@@ -305,9 +335,6 @@ __device__ __forceinline__ void strip_march(const StripInst &m, int par, int xb,
         for (int a = 1; a < NQ; a++) fn[a] = row_f(slot, a);
         strip_boundary<D>(F, out, fn, b0, rho, ux, uy, m, side, on0, on1);
     };
-    // F +- the signed flux
-    auto minus = [](float2 F, float2 fl, int sg) { return sg > 0 ? sub2(F, fl) : __fadd2_rn(F, fl); };
-    auto plus = [](float2 F, float2 fl, int sg) { return sg > 0 ? __fadd2_rn(F, fl) : sub2(F, fl); };
 
     const int js = (y0 == 0 && !pery) ? 0 : y0 - 1, je = (y1 == ny && !pery) ? ny - 1 : y1;   // rows processed
     const bool below = pery || js > 0;
@@ -387,7 +414,7 @@ __device__ __forceinline__ void strip_march(const StripInst &m, int par, int xb,
                 strip_face<1>(yf, v, t0, t1, t3, m);
                 if (j > y0) {
 #pragma unroll
-                    for (int q = 0; q < 6; q++) F[YSLOT_A(q)] = plus(F[YSLOT_A(q)], yf[q], EY(YSLOT_A(q)));
+                    for (int q = 0; q < 6; q++) F[YSLOT_A(q)] = strip_plus(F[YSLOT_A(q)], yf[q], EY(YSLOT_A(q)));
                     update(s0, j > 0 ? j - 1 : ny - 1, F);
                 }
             } else {
@@ -421,7 +448,7 @@ __device__ __forceinline__ void strip_march(const StripInst &m, int par, int xb,
                     float2 fl[6];
 #pragma unroll
                     for (int q = 0; q < 6; q++) {
-                        const float2 n = minus(dup(0.0f), xf[q], EX(XSLOT_A(q)));
+                        const float2 n = strip_minus(dup(0.0f), xf[q], EX(XSLOT_A(q)));
                         fl[q] = make_float2(xf[q].y, __shfl_down_sync(0xffffffffu, xf[q].x, 1));
                         F[XSLOT_A(q)] = make_float2(hW0 ? n.x : 0.0f, n.y);
                     }
@@ -432,7 +459,7 @@ __device__ __forceinline__ void strip_march(const StripInst &m, int par, int xb,
                     }
 #pragma unroll
                     for (int q = 0; q < 6; q++) {
-                        const float2 p = plus(F[XSLOT_A(q)], fl[q], EX(XSLOT_A(q)));
+                        const float2 p = strip_plus(F[XSLOT_A(q)], fl[q], EX(XSLOT_A(q)));
                         if (hE0) F[XSLOT_A(q)].x = p.x;
                         if (hE1) F[XSLOT_A(q)].y = p.y;
                     }
@@ -451,7 +478,7 @@ __device__ __forceinline__ void strip_march(const StripInst &m, int par, int xb,
                 }
                 if (hS) {
 #pragma unroll
-                    for (int q = 0; q < 6; q++) F[YSLOT_A(q)] = minus(F[YSLOT_A(q)], yf[q], EY(YSLOT_A(q)));
+                    for (int q = 0; q < 6; q++) F[YSLOT_A(q)] = strip_minus(F[YSLOT_A(q)], yf[q], EY(YSLOT_A(q)));
                 } else {
                     boundary(std::integral_constant<int, 3>{}, s1, 0, F, yf, true, true);
                 }

@@ -330,14 +330,14 @@ def autotune_clear():
 class BatchStatus(C.Structure):
     _fields_ = [("instances", C.c_int64), ("cells", C.c_int64), ("items", C.c_int64), ("pool_bytes", C.c_int64),
                 ("pool_used", C.c_int64), ("steps", C.c_int64), ("grid", C.c_int32), ("ctas_per_sm", C.c_int32),
-                ("graph_steps", C.c_int32), ("precision", C.c_int32), ("per_item", C.c_int32)]
+                ("graph_steps", C.c_int32), ("precision", C.c_int32), ("per_item", C.c_int32), ("march", C.c_int32)]
 
     def as_dict(self):
         return {k: getattr(self, k) for k, _ in self._fields_}
 
 
 class Batch:
-    """sdugks_batch: many uniform-grid solves advanced by one batched kernel per step."""
+    """sdugks_batch: many uniform-grid solves advanced together, step by step."""
 
     def __init__(self, pool_bytes: int, precision="fp32", max_instances: int = 1024, stream=None):
         L = lib()
