@@ -355,8 +355,10 @@ def roofline_of(info, precision, n, launch_ms, key):
     alg_bytes = (STATE_BYTES[precision] + mesh_b) * n
     achieved = alg_bytes / (launch_ms / 1e3) / 1e9
     kname = {1: "k_step_tiled", 2: "k_step_cart"}[info["kernel"]]
-    if kname == "k_step_cart" and precision == "fp32" and n >= 448 * 448:
-        kname = "k_step_strip"           # large FP32 grids march
+    if info["march"]:
+        kname = "k_step_strip"
+    elif kname == "k_step_cart" and precision == "fp64" and info["staging"] == 0:
+        kname = "k_step_cart64"
     resident = (STATE_BYTES[precision] + mesh_b) * n < 0.8 * L2_BYTES
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "traffic": profiled_traffic(key), "kernel": kname, "algorithmic_bytes_per_launch": alg_bytes,

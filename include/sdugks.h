@@ -109,7 +109,7 @@ typedef struct sdugks_params {
 /* What a solver chose and holds (sdugks_solver_info). */
 typedef struct sdugks_info {
     int64_t n_cells, n_faces;     /* after periodic faces are merged pairwise          */
-    int64_t n_tiles;              /* tiles (blocks) of the grid: CTAs of a block or tile step */
+    int64_t n_tiles;              /* tiles, or blocks of tile_cells cells, of the grid (see step_ctas) */
     int64_t halo_cells;           /* summed over tiles (ring 1 + ring 2)               */
     int64_t steps_done;           /* steps since init / set_state                      */
     int64_t device_bytes;         /* device memory held by the solver                  */
@@ -117,7 +117,7 @@ typedef struct sdugks_info {
     double mesh_bytes_per_cell_step;  /* mesh data the kernel reads per cell and step  */
     int32_t kernel;               /* SDUGKS_KERNEL_TILED or SDUGKS_KERNEL_CARTESIAN    */
     int32_t precision;
-    int32_t tile_cells;
+    int32_t tile_cells;           /* as requested, or the general choice for the grid size */
     int32_t nx, ny;               /* Cartesian kernel: grid size, else 0               */
     int32_t staging;              /* SDUGKS_STAGING_* in use                           */
     int32_t one_code_path;        /* Cartesian kernel: 1 when the grid runs in one wave and
@@ -125,6 +125,11 @@ typedef struct sdugks_info {
                                      blocks take the compile-time interior variant      */
     int64_t n_boundary_faces;     /* faces on non-periodic patches: the rows of
                                      sdugks_step_boundary_flux                          */
+    /* what sdugks_step launches, which can differ from tile_cells and n_tiles where the tile
+     * size was left open */
+    int64_t step_ctas;            /* CTAs of a step's launch (in a graph)              */
+    int32_t step_cells;           /* cells of its blocks or tiles, at most; 0 if it marches */
+    int32_t march;                /* 1: steps by marching warps (FP32 grids of many waves) */
 } sdugks_info;
 
 /* ---- mesh ---------------------------------------------------------------------- */

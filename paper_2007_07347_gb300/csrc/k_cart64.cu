@@ -382,7 +382,7 @@ template <int BX, int BY> int64_t cost64(int nx, int ny, int n_sm)
 
 }  // namespace
 
-int cart64_shape(int nx, int ny, int n_sm)
+int cart64_shape(int nx, int ny, int n_sm)          // an index of CART64_BLOCK
 {
     const int64_t c[3] = {cost64<16, 14>(nx, ny, n_sm), cost64<8, 8>(nx, ny, n_sm), cost64<4, 4>(nx, ny, n_sm)};
     return c[0] <= c[1] && c[0] <= c[2] ? 0 : (c[1] <= c[2] ? 1 : 2);

@@ -385,6 +385,8 @@ struct sdugks_solver {
     int cart_shape = 0;             // Cartesian block shape (CART_TY)
     int launch_shape = 0;           // the shape given to the launch: cart_shape, or FP64's own (cart64_shape)
     CartTma *tma = nullptr;         // Cartesian: tensor maps of the TMA staging (nullptr: plain loads)
+    int64_t step_ctas = 0;          // of an ordinary step's launch, and the cells of its blocks or tiles
+    int32_t step_cells = 0;
     StripInst strip{};              // Cartesian: the solve as the marching form sees it
     int strip_rows = 0;             // rows per warp of the marching form (0: blocks)
     bool strip_early = true;
@@ -740,6 +742,13 @@ static int create_cart(const sdugks_mesh &m, const CartGrid &g, const sdugks_par
             }
         }
         s->ci.early = early_start(ctas, slots, n_sm);
+        s->step_ctas = ctas;
+        s->step_cells = 16 * CART_TY[s->launch_shape];
+        if (prec == P_FP64 && !use_tma) {
+            const int *b = CART64_BLOCK[s->launch_shape];
+            s->step_ctas = (int64_t)((g.nx + b[0] - 1) / b[0]) * ((g.ny + b[1] - 1) / b[1]);
+            s->step_cells = b[0] * b[1];
+        }
     }
     // FP32 grids of many waves march (step_strip.cuh) where the two models say that it is
     // faster: 1.95 us per unit of strip_rows' cost against 54 ps per cell of the blocks'
@@ -758,8 +767,9 @@ static int create_cart(const sdugks_mesh &m, const CartGrid &g, const sdugks_par
         fill_strip(s->ci, s->strip);
         int n_sm = 1;
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, s->device);
-        s->strip_early = early_start((int64_t)strip_count(g.nx, g.px) * ((g.ny + s->strip_rows - 1) / s->strip_rows),
-                                     strip_slots(), n_sm);
+        s->step_ctas = (int64_t)strip_count(g.nx, g.px) * ((g.ny + s->strip_rows - 1) / s->strip_rows);
+        s->step_cells = 0;
+        s->strip_early = early_start(s->step_ctas, strip_slots(), n_sm);
     }
     // interior blocks staged by tensor copies; the maps hold the fixed addresses of the
     // two state buffers
@@ -1176,6 +1186,8 @@ extern "C" int sdugks_solver_create(const sdugks_mesh *m, const sdugks_params *p
     s->n_bfaces = n_bfaces;
     s->stream = static_cast<cudaStream_t>(stream);
     s->n = n; s->npad = npad; s->nf = F.nf; s->n_tiles = nt; s->halo_cells = halo_total;
+    s->step_ctas = nt;
+    for (const auto &t : final_tiles) s->step_cells = std::max(s->step_cells, (int32_t)(t.second - t.first));
     s->kernel = SDUGKS_KERNEL_TILED;
     const size_t fs = prec == P_FP64 ? 8 : (prec == P_FP32 ? 4 : 2);
     s->n_red_blocks = residual_blocks(n);
@@ -1638,6 +1650,9 @@ extern "C" int sdugks_solver_info(const sdugks_solver *s, sdugks_info *o)
     o->staging = s->tma ? SDUGKS_STAGING_TMA : SDUGKS_STAGING_LOADS;
     o->n_boundary_faces = s->n_bfaces;
     o->one_code_path = s->cart_general ? 1 : 0;
+    o->step_ctas = s->step_ctas;
+    o->step_cells = s->step_cells;
+    o->march = s->strip_rows > 0 ? 1 : 0;
     return SDUGKS_OK;
 }
 

@@ -152,6 +152,7 @@ int cart_shape_occupancy(int prec, int shape, bool tma);   // resident CTAs per 
 cudaError_t prepare_cart64();
 cudaError_t launch_step_cart64(const CartInst &m, int shape, int parity, cudaStream_t st);
 int cart64_shape(int nx, int ny, int n_sm);
+constexpr int CART64_BLOCK[3][2] = {{16, 14}, {8, 8}, {4, 4}};
 // One uniform-grid solve as the marching form sees it (FP32 storage; no symmetry side,
 // an even nx where x is periodic): the grid and its side rules, the ping-pong state, and
 // the step's constants, each twice (one operand of a paired instruction).

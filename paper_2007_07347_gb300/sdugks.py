@@ -52,7 +52,8 @@ class Info(C.Structure):
                 ("steps_done", C.c_int64), ("device_bytes", C.c_int64), ("state_bytes_per_cell_step", C.c_double),
                 ("mesh_bytes_per_cell_step", C.c_double), ("kernel", C.c_int32), ("precision", C.c_int32),
                 ("tile_cells", C.c_int32), ("nx", C.c_int32), ("ny", C.c_int32), ("staging", C.c_int32),
-                ("one_code_path", C.c_int32), ("n_boundary_faces", C.c_int64)]
+                ("one_code_path", C.c_int32), ("n_boundary_faces", C.c_int64), ("step_ctas", C.c_int64),
+                ("step_cells", C.c_int32), ("march", C.c_int32)]
 
     def as_dict(self):
         return {k: getattr(self, k) for k, _ in self._fields_}

@@ -1,0 +1,38 @@
+"""sdugks_solver_info says what a step launches, also where the tile size was left open."""
+import pytest
+
+from paper_2007_07347_gb300 import meshes as M
+
+pytestmark = pytest.mark.gpu
+
+BLOCK = {16: (4, 4), 64: (8, 8), 128: (16, 8), 224: (16, 14), 256: (16, 16)}
+
+
+def _info(case, precision, **kw):
+    from paper_2007_07347_gb300 import sdugks as S
+    return S.Solver.from_case(case, precision, **kw).info()
+
+
+@pytest.mark.parametrize("precision,n,cells,staging", [
+    ("fp64", 20, (16,), "loads"), ("fp64", 130, (64, 224), "loads"), ("fp64", 300, (224,), "loads"), ("fp64", 60, (256,), "tma"),
+    ("fp32", 100, (128,), "loads"), ("fp32", 256, (224,), "loads"), ("fp32", 100, (128, 224, 256), "tma"),
+    ("bf16dev", 300, (128, 224, 256), "loads")])
+def test_block_steps(precision, n, cells, staging):
+    i = _info(M.cavity(n), precision, staging=staging)
+    assert i["march"] == 0 and i["step_cells"] in cells
+    bx, by = BLOCK[i["step_cells"]]
+    assert i["step_ctas"] == -(-n // bx) * -(-n // by)
+
+
+def test_marching_steps():
+    i = _info(M.cavity(700), "fp32")
+    assert i["march"] == 1 and i["step_cells"] == 0
+    assert i["step_ctas"] % 12 == 0                        # twelve strips of 60 columns
+    assert _info(M.cavity(700), "fp32", staging="tma")["march"] == 0
+
+
+def test_tile_steps():
+    case = M.cylinder(96, 48, first=0.01, r_far=10.0, shuffle_seed=1)
+    for kw, most in ((dict(), 64), (dict(tile_cells=128), 128), (dict(tile_cells=100), 100)):
+        i = _info(case, "fp32", **kw)
+        assert most // 2 < i["step_cells"] <= most and i["step_ctas"] == i["n_tiles"] >= 96 * 48 // most
