@@ -743,7 +743,7 @@ static int create_cart(const sdugks_mesh &m, const CartGrid &g, const sdugks_par
         }
         s->ci.early = early_start(ctas, slots, n_sm);
         s->step_ctas = ctas;
-        s->step_cells = 16 * CART_TY[s->launch_shape];
+        s->step_cells = 16 * CART_TY[use_tma ? s->cart_shape : s->launch_shape];
         if (prec == P_FP64 && !use_tma) {
             const int *b = CART64_BLOCK[s->launch_shape];
             s->step_ctas = (int64_t)((g.nx + b[0] - 1) / b[0]) * ((g.ny + b[1] - 1) / b[1]);
