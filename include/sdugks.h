@@ -91,10 +91,10 @@ typedef struct sdugks_params {
                             bf16 and fp16 storage): 256, 224 or 128 for 16x16, 16x14 or 16x8 blocks;
                             0 = chosen from the grid size (Cartesian) or 128 (tiled; meshes
                             that fill less than half the device run on half tiles, in the
-                            same cell order).  With
-                            plain loads, FP32 grids of many waves of blocks (about 430^2
-                            cells and up, no symmetry side) are stepped by marching warps
-                            instead; the blocks then run the diagnostic steps only */
+                            same cell order).  With 0 and plain loads, FP32 grids of many
+                            waves of blocks (about 430^2 cells and up, no symmetry side) are
+                            stepped by marching warps; blocks then run the diagnostic
+                            steps only.  See sdugks_info.step_cells and .march */
     int32_t graph_steps; /* steps per captured CUDA graph in sdugks_step, 0 = auto, <0 = off */
     int32_t staging;     /* SDUGKS_STAGING_*; TMA requires the Cartesian kernel (else
                             INVALID_ARG).  A TMA copy that does not land within the wait

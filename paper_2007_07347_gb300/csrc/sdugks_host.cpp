@@ -750,11 +750,11 @@ static int create_cart(const sdugks_mesh &m, const CartGrid &g, const sdugks_par
             s->step_cells = b[0] * b[1];
         }
     }
-    // FP32 grids of many waves march (step_strip.cuh) where the two models say that it is
-    // faster: 1.95 us per unit of strip_rows' cost against 54 ps per cell of the blocks'
+    // FP32 grids of many waves march (step_strip.cuh), unless a block is asked for by its size, where
+    // the two models say that it is faster: 1.95 us per unit of strip_rows' cost against 54 ps per cell of the blocks'
     // (16x8, padding included).  GB300, FP32 cavity, blocks / marching in us per step: 384^2
     // 8.1 / 9.8, 448^2 11.3 / 9.8, 512^2 14.0 / 11.3, 1024^2 48.8 / 34.2, 2048^2 181 / 112.
-    if (!use_tma && !s->cart_general && strip_fits(s->ci, prec)) {
+    if (!use_tma && prm->tile_cells == 0 && !s->cart_general && strip_fits(s->ci, prec)) {
         const int strips = strip_count(g.nx, g.px);
         double cost = 0.0;
         const int rows = strip_rows(strip_slots(), g.ny, [&](int r) { return (int64_t)strips * ((g.ny + r - 1) / r); }, cost);
@@ -1759,11 +1759,13 @@ extern "C" int sdugks_autotune(const sdugks_mesh *m, const sdugks_params *base, 
     sdugks_params p0 = *base;
     p0.tile_cells = 0; p0.graph_steps = 0; p0.staging = SDUGKS_STAGING_LOADS;
     int32_t kernel = 0;
+    bool march = false;
     {
         sdugks_solver *s = nullptr;
         int rc = sdugks_solver_create(m, &p0, stream, &s);
         if (rc) return rc;
         kernel = s->kernel;
+        march = s->strip_rows > 0;
         sdugks_solver_destroy(s);
     }
     std::vector<int32_t> tiles, stagings{SDUGKS_STAGING_LOADS};
@@ -1771,6 +1773,7 @@ extern "C" int sdugks_autotune(const sdugks_mesh *m, const sdugks_params *base, 
         stagings.push_back(SDUGKS_STAGING_TMA);
         if (base->precision == P_FP64) tiles = {0};
         else tiles = {256, 224, 128};
+        if (march) tiles.insert(tiles.begin(), 0);
     } else {
         tiles = {64, 96, 108, 120, 128};
     }
@@ -1782,6 +1785,7 @@ extern "C" int sdugks_autotune(const sdugks_mesh *m, const sdugks_params *base, 
     for (int32_t t : tiles)
         for (int32_t sg : stagings)
             for (int32_t g : graphs) {
+                if (march && t == 0 && sg != SDUGKS_STAGING_LOADS) continue;       // blocks of the general choice: one of the others
                 sdugks_params p = p0;
                 p.kernel = kernel;
                 p.tile_cells = t;

@@ -36,3 +36,17 @@ def test_tile_steps():
     for kw, most in ((dict(), 64), (dict(tile_cells=128), 128), (dict(tile_cells=100), 100)):
         i = _info(case, "fp32", **kw)
         assert most // 2 < i["step_cells"] <= most and i["step_ctas"] == i["n_tiles"] >= 96 * 48 // most
+
+
+def test_a_block_asked_for_by_its_size_is_run():
+    """tile_cells = 0 marches on a large grid; 256, 224 and 128 are those blocks, so that the autotuner's
+    candidates are different launches, with marching among them."""
+    from paper_2007_07347_gb300 import sdugks as S
+    case = M.cavity(640)
+    for cells in (256, 224, 128):
+        i = _info(case, "fp32", tile_cells=cells)
+        assert i["march"] == 0 and i["step_cells"] == cells
+    S.autotune_clear()
+    s = S.Solver.tuned(case, "fp32", steps=64)
+    assert s.tune["candidates"] == (1 + 3 * 2) * 3 and s.tune["tile_cells"] in (0, 128, 224, 256)
+    assert s.info()["march"] == int(s.tune["tile_cells"] == 0)
