@@ -386,9 +386,9 @@ int sdugks_batch_get_macros(sdugks_batch *b, int64_t id, double *rho, double *u)
 
 /* Time `steps` steps of each candidate launch form and keep the fastest: one CTA per
  * work item (the default), or a fixed grid of 1, 2 or 4 times the resident CTAs that
- * walks the work list (see sdugks_batch_status.per_item and .grid; instances stepped
- * by marching warps have one form).  Call with
- * instances admitted.  With one CTA per item, the step graph is captured again after
+ * walks the work list (see sdugks_batch_status.per_item and .grid).  Call with
+ * instances admitted.  FP32 instances without a symmetry side or an odd periodic width have
+ * one form: where there are no others, this returns without a step.  With one CTA per item, the step graph is captured again after
  * the item count changes (instances admitted or removed). */
 int sdugks_batch_autotune(sdugks_batch *b, int64_t steps);
 

@@ -2299,6 +2299,7 @@ extern "C" int sdugks_batch_autotune(sdugks_batch *b, int64_t steps)
 {
     if (!b || steps <= 0) return fail(SDUGKS_ERR_INVALID_ARG, "bad argument");
     if (b->inst.empty()) return fail(SDUGKS_ERR_STATE, "autotune needs admitted instances");
+    if (b->n_block == 0) return SDUGKS_OK;      // one form: every candidate would be the same launches
     CUDA_TRY(cudaSetDevice(b->device));
     cudaEvent_t e0, e1;
     CUDA_TRY(cudaEventCreate(&e0));

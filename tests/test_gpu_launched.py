@@ -50,3 +50,18 @@ def test_a_block_asked_for_by_its_size_is_run():
     s = S.Solver.tuned(case, "fp32", steps=64)
     assert s.tune["candidates"] == (1 + 3 * 2) * 3 and s.tune["tile_cells"] in (0, 128, 224, 256)
     assert s.info()["march"] == int(s.tune["tile_cells"] == 0)
+
+
+def test_batch_autotune_without_a_choice_changes_nothing():
+    """Only instances with one form: the launch form for others stays one CTA per item, and no step is made.
+    With one that walks or not (a symmetry side) it is timed."""
+    from paper_2007_07347_gb300 import sdugks as S
+    b = S.Batch(64 << 20, "fp32", max_instances=4)
+    i = b.add_case(M.cavity(40, Re=100.0))
+    b.autotune(4)
+    assert b.info()["per_item"] == 1 and b.residual()[i][2] == 0
+    mesh = M.cartesian(40, 20, 40.0, 20.0)
+    b.add_case(M.Case("mirror", mesh, [(3, M.BC_WALL, (0, 0, 0)), (1, M.BC_WALL, (0, 0, 0)), (0, M.BC_MOVING_WALL, (0.05, 0, 0)),
+                                       (2, M.BC_SYMMETRY, (0, 0, 0))], tau=0.05, dt=0.25))
+    b.autotune(4)
+    assert b.residual()[i][2] == 4 * 10
