@@ -1,9 +1,8 @@
 """In-tree build of libsdugks.so for sm_103a (nvcc + g++, no cmake).
 
 The CUDA translation units are compiled in parallel with
-``-gencode arch=compute_103a,code=sm_103a``; the FP64 units of the tiled step and of the
-TMA staging additionally with ``--fmad=false``, so that their FP64 arithmetic rounds every
-product and sum.
+``-gencode arch=compute_103a,code=sm_103a``; the FP64 unit of the tiled step additionally
+with ``--fmad=false``, so that its FP64 arithmetic rounds every product and sum.
 """
 from __future__ import annotations
 
@@ -25,7 +24,6 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CU_UNITS = {
     "k_step_fp64.cu": ["--fmad=false"],
     "k_step_fp32.cu": [],
-    "k_cart_fp64.cu": ["--fmad=false"],
     "k_cart64.cu": [],
     "k_cart.cu": [],
     "k_strip.cu": [],

@@ -1,15 +1,11 @@
 // k_cart.cu -- FP32-compute instances of the Cartesian fused step by blocks, and the choice
-// of the kernel: FP64 runs on k_cart64.cu, or with TMA staging on the FP64 instance of
-// k_cart_fp64.cu (its own unit, --fmad=false).
+// of the kernel: FP64 runs on k_cart64.cu.
 #include "step_cart.cuh"
 
 namespace sdugks {
 
 // Block shapes of the FP32-compute instances: 16 x TY with TY in {16, 14, 8}
 // (shape index 0, 1, 2).  FP64 with TMA staging uses 16 x 16 only.
-
-cudaError_t prepare_cart_fp64();
-cudaError_t launch_cart_fp64_tma(const CartInst &m, const CartTma &tma, int parity, cudaStream_t st);
 
 template <int P> cudaError_t prepare_shapes()
 {
@@ -21,10 +17,7 @@ template <int P> cudaError_t prepare_shapes()
 
 cudaError_t prepare_cart(int prec)
 {
-    if (prec == P_FP64) {
-        const cudaError_t e = prepare_cart64();
-        return e == cudaSuccess ? prepare_cart_fp64() : e;
-    }
+    if (prec == P_FP64) return prepare_cart64();
     if (prec == P_FP16DEV) return prepare_shapes<P_FP16DEV>();
     return prec == P_BF16DEV ? prepare_shapes<P_BF16DEV>() : prepare_shapes<P_FP32>();
 }
@@ -41,7 +34,7 @@ cudaError_t launch_step_cart(int prec, int shape, const CartInst &m, const CartT
                              cudaStream_t st)
 {
     if (prec == P_FP64)         // diagnostic steps run with plain loads; shape: cart64_shape's
-        return tma && !(m.force || m.bface) ? launch_cart_fp64_tma(m, *tma, parity, st) : launch_step_cart64(m, shape, parity, st);
+        return tma && !(m.force || m.bface) ? launch_step_cart64_tma(m, *tma, parity, st) : launch_step_cart64(m, shape, parity, st);
     if (prec == P_BF16DEV) return launch_shape<P_BF16DEV>(shape, m, tma, general, parity, st);
     if (prec == P_FP16DEV) return launch_shape<P_FP16DEV>(shape, m, tma, general, parity, st);
     return launch_shape<P_FP32>(shape, m, tma, general, parity, st);

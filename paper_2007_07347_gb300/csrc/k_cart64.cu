@@ -167,16 +167,14 @@ __device__ __forceinline__ void boundary64(double flux[6], const double *f, int 
     }
 }
 
-template <int BX, int BY, bool DIAG>
-__global__ void __launch_bounds__(Shape64<BX, BY>::NT, Shape64<BX, BY>::CTAS)
-k_step_cart64(const CartInst m, const Cart64K k, int par)
+// One block; s_f: shared memory of Shape64::SMEM bytes.  BOX (blocks whose ring lies inside the
+// grid): f^n of the block and its ring has been copied to s_f, and W^n to where the fluxes go later.
+template <int BX, int BY, bool DIAG, bool BOX>
+__device__ __forceinline__ void cart64_block(const CartInst &m, const Cart64K &k, int par, double *s_f)
 {
     using Sh = Shape64<BX, BY>;
     constexpr int LX = Sh::LX, LY = Sh::LY, LP = Sh::LP, NT = Sh::NT;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    double *const s_f = reinterpret_cast<double *>(smem_raw);     // [NQ][LY][LX]
-    double *const s_fx = s_f + NQ * LP, *const s_fy = s_fx + 6 * Sh::NXF;
-    step_dependency_wait();
+    double *const s_fx = s_f + NQ * LP, *const s_fy = s_fx + 6 * Sh::NXF;      // s_f [NQ][LY][LX]
     const double *__restrict__ fin = static_cast<const double *>(m.f[par]);
     double *__restrict__ fout = static_cast<double *>(m.f[1 - par]);
     const double *__restrict__ Wn = m.W[par];
@@ -192,12 +190,12 @@ k_step_cart64(const CartInst m, const Cart64K k, int par)
     for (int p = tid; p < LP; p += NT) {
         int gi = x0 + p % LX - 2, gj = y0 + p / LX - 2, mir = 0;
         bool in = true;
-        if (gi < 0 || gi >= nx) {
+        if (!BOX && (gi < 0 || gi >= nx)) {
             if (px) { gi %= nx; if (gi < 0) gi += nx; }
             else if (gi < 0 ? symL : symR) { gi = gi < 0 ? -1 - gi : 2 * nx - 1 - gi; mir |= 1; }
             in = gi >= 0 && gi < nx;
         }
-        if (gj < 0 || gj >= ny) {
+        if (!BOX && (gj < 0 || gj >= ny)) {
             if (py) { gj %= ny; if (gj < 0) gj += ny; }
             else if (gj < 0 ? symB : symT) { gj = gj < 0 ? -1 - gj : 2 * ny - 1 - gj; mir |= 2; }
             in = in && gj >= 0 && gj < ny;
@@ -205,9 +203,11 @@ k_step_cart64(const CartInst m, const Cart64K k, int par)
         if (!in) continue;
         const int64_t g = gi + pitch * gj;
         double fv[NQ], fe[NQ];
-        const double w0 = Wn[g], w1 = Wn[np + g], w2 = Wn[2 * np + g];
+        const double *const w = BOX ? s_fx + p : Wn + g, *const fs = BOX ? s_f + p : fin + g;
+        const int64_t ws = BOX ? LP : np;
+        const double w0 = w[0], w1 = w[ws], w2 = w[2 * ws];
 #pragma unroll
-        for (int a = 0; a < NQ; a++) fv[a] = fin[a * np + g];
+        for (int a = 0; a < NQ; a++) fv[a] = fs[a * ws];
         const double iv = recip64(w0);
         feq64<true>(k.b * w0, w1 * iv, w2 * iv, fe);
 #pragma unroll
@@ -330,6 +330,46 @@ k_step_cart64(const CartInst m, const Cart64K k, int par)
     for (int a = 0; a < NQ; a++) fout[a * np + g] = fma(k.inv, a == 0 ? fn[a] : fn[a] - F[a], fe[a]);
 }
 
+template <int BX, int BY, bool DIAG>
+__global__ void __launch_bounds__(Shape64<BX, BY>::NT, Shape64<BX, BY>::CTAS)
+k_step_cart64(const CartInst m, const Cart64K k, int par)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    step_dependency_wait();
+    cart64_block<BX, BY, DIAG, false>(m, k, par, reinterpret_cast<double *>(smem_raw));
+}
+
+// TMA staging: f^n and W^n of the blocks whose ring lies inside the grid come by two tensor
+// copies (tf, tw: the maps of buffer par), f^n straight to where its fbar+ goes, each thread replacing
+// what it read.  The arithmetic is that of the other blocks: the same bits as with plain loads.
+using Sh64T = Shape64<16, 16>;
+static_assert(CartTmaBox<P_FP64, 16, 16>::F_BYTES == sizeof(double) * NQ * Sh64T::LP, "the f box is s_f");
+static_assert(CartTmaBox<P_FP64, 16, 16>::F_BYTES % 128 == 0, "the W box starts on a 128-byte boundary");
+static_assert(CartTmaBox<P_FP64, 16, 16>::W_BYTES <= sizeof(double) * 6 * (Sh64T::NXF + Sh64T::NYF), "the W box fits the fluxes' place");
+constexpr size_t SMEM64T = Sh64T::SMEM + 16 + 128;           // the barrier; 128 bytes of slack align the base
+__global__ void __launch_bounds__(Sh64T::NT, Sh64T::CTAS)
+k_step_cart64_tma(const CartInst m, const Cart64K k, int par, const __grid_constant__ CUtensorMap tf,
+                  const __grid_constant__ CUtensorMap tw)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    step_dependency_wait();
+    uint32_t sa;
+    unsigned char *const sm = aligned_smem(smem_raw, sa);
+    double *const s_f = reinterpret_cast<double *>(sm);
+    if (cart_block_interior<16, 16>(m, blockIdx.x, blockIdx.y)) {
+        const uint32_t bar = sa + (uint32_t)Sh64T::SMEM;
+        if (threadIdx.x == 0) mbar_init(bar);
+        __syncthreads();
+        if (threadIdx.x == 0)
+            tma_issue_block<P_FP64, 16, 16>(bar, sa, sa + (uint32_t)CartTmaBox<P_FP64, 16, 16>::F_BYTES, &tf, &tw,
+                                            blockIdx.x * 16, blockIdx.y * 16);
+        if (!cta_wait_staged(m, bar, 0)) return;
+        cart64_block<16, 16, false, true>(m, k, par, s_f);
+    } else {
+        cart64_block<16, 16, false, false>(m, k, par, s_f);
+    }
+}
+
 Cart64K coefs64(const CartInst &m)
 {
     Cart64K k;
@@ -393,7 +433,16 @@ cudaError_t prepare_cart64()
     cudaError_t e = prepare64<16, 14>();
     if (e == cudaSuccess) e = prepare64<8, 8>();
     if (e == cudaSuccess) e = prepare64<4, 4>();
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_step_cart64_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM64T);
     return e;
+}
+
+cudaError_t launch_step_cart64_tma(const CartInst &m, const CartTma &tma, int parity, cudaStream_t st)
+{
+    const dim3 grid((m.nx + 15) / 16, (m.ny + 15) / 16);
+    return launch_step_kernel(false, k_step_cart64_tma, grid, dim3(Sh64T::NT), SMEM64T, st, m, coefs64(m), parity,
+                              tma.f[parity], tma.W[parity]);
 }
 
 cudaError_t launch_step_cart64(const CartInst &m, int shape, int parity, cudaStream_t st)

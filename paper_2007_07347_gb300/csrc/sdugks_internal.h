@@ -148,8 +148,9 @@ cudaError_t make_cart_tma(int prec, int shape, const CartInst &m, CartTma &out);
 cudaError_t launch_step_cart(int prec, int shape, const CartInst &m, const CartTma *tma, bool general, int parity,
                              cudaStream_t st);
 int cart_shape_occupancy(int prec, int shape, bool tma);   // resident CTAs per SM
-// FP64 with plain loads: blocks of 16x14, 8x8 or 4x4 cells (shape 0, 1, 2), by grid size
+// FP64: blocks of 16x14, 8x8 or 4x4 cells (shape 0, 1, 2), by grid size; 16x16 with TMA staging
 cudaError_t prepare_cart64();
+cudaError_t launch_step_cart64_tma(const CartInst &m, const CartTma &tma, int parity, cudaStream_t st);
 cudaError_t launch_step_cart64(const CartInst &m, int shape, int parity, cudaStream_t st);
 int cart64_shape(int nx, int ny, int n_sm);
 constexpr int CART64_BLOCK[3][2] = {{16, 14}, {8, 8}, {4, 4}};

@@ -147,13 +147,6 @@ __device__ constexpr int YSLOT_A(int k) { return k == 0 ? 2 : k == 1 ? 4 : k == 
 
 // Step coefficients in the compute precision.
 template <class R> struct CartK;
-template <> struct CartK<double> {
-    double a, b, c, r, dt, dtV, hx, hy, ihx, ihy;
-    __device__ explicit CartK(const CartInst &m)
-        : a(m.a), b(m.b), c(m.c), r(m.r), dt(m.dt), dtV(m.dtV), hx(m.dx), hy(m.dy), ihx(m.ihx), ihy(m.ihy) {}
-    __device__ static double par(const CartInst &m, int side, int i) { return m.side_par[side][i]; }
-    __device__ static double drho_par(const CartInst &m, int side) { return m.side_par[side][0] - 1.0; }
-};
 template <> struct CartK<float> {
     float a, b, c, r, dt, dtV, hx, hy, ihx, ihy;
     __device__ explicit CartK(const CartInst &m)
@@ -185,51 +178,12 @@ __device__ __forceinline__ R cart_extrap(const R *s_fbp, int l, const Sten<R> &s
     return v;
 }
 
-// Interface distribution on a face between cell L (below/left) and R (above/right),
-// along axis AX (0: face of constant x, 1: of constant y), from the staged fbar+ of
-// the two cells and their neighbours; writes (xi . n_+ l) f_b of the six crossing
-// velocities (n_+ = +x or +y).
-template <int AX, class R>
-__device__ __forceinline__ void cart_interior_face(R flux[6], const R *s_fbp, int lL, int lR, const Sten<R> &sL,
-                                                   const Sten<R> &sR, const CartK<R> &k, int LXY)
-{
-    // x_f - x_L = +h/2 along the axis, x_f - x_R = -h/2
-    const R hl = AX == 0 ? R(0.5) * k.hx : R(0.5) * k.hy;
-    R fbar[NQ], w0 = R(0), w1 = R(0), w2 = R(0);
-#define SDUGKS_FACE_ALPHA(a)                                                                        \
-    {                                                                                               \
-        constexpr int sg = AX == 0 ? EX(a) : EY(a);   /* sign of xi . n_+ */                        \
-        const R ex = R(EX(a)) * k.dt, ey = R(EY(a)) * k.dt;                                         \
-        R A = R(0), B = R(0);                                                                       \
-        constexpr bool ux = AX == 0 || EX(a) != 0, uy = AX == 1 || EY(a) != 0;                     \
-        if (sg >= 0) A = cart_extrap<a, ux, uy, R>(s_fbp, lL, sL, AX == 0 ? hl - ex : -ex, AX == 0 ? -ey : hl - ey, LXY); \
-        if (sg <= 0) B = cart_extrap<a, ux, uy, R>(s_fbp, lR, sR, AX == 0 ? -hl - ex : -ex, AX == 0 ? -ey : -hl - ey, LXY); \
-        fbar[a] = sg > 0 ? A : (sg < 0 ? B : R(0.5) * (A + B));                                     \
-        w0 += fbar[a];                                                                              \
-        if (EX(a) == 1) w1 += fbar[a]; else if (EX(a) == -1) w1 -= fbar[a];                         \
-        if (EY(a) == 1) w2 += fbar[a]; else if (EY(a) == -1) w2 -= fbar[a];                         \
-    }
-    SDUGKS_FACE_ALPHA(0) SDUGKS_FACE_ALPHA(1) SDUGKS_FACE_ALPHA(2) SDUGKS_FACE_ALPHA(3) SDUGKS_FACE_ALPHA(4)
-    SDUGKS_FACE_ALPHA(5) SDUGKS_FACE_ALPHA(6) SDUGKS_FACE_ALPHA(7) SDUGKS_FACE_ALPHA(8)
-#undef SDUGKS_FACE_ALPHA
-    R ux, uy, feqb[NQ];
-    vel_of<R>(w0, w1, w2, ux, uy);
-    feq9f<R>(w0, ux, uy, feqb);
-    const R len = AX == 0 ? k.hy : k.hx;
-#pragma unroll
-    for (int q = 0; q < 6; q++) {
-        const int a = AX == 0 ? XSLOT_A(q) : YSLOT_A(q);
-        const int sg = AX == 0 ? EX(a) : EY(a);
-        const R s = sg > 0 ? len : -len;
-        flux[q] = s * ((fbar[a] + k.b * feqb[a]) * k.c);
-    }
-}
-
-// FP32 specialisation of cart_interior_face with paired arithmetic: on this GPU one
-// FFMA2/FMUL2 instruction does two independent FP32 operations (each rounded as the
-// scalar operation), so the reconstructions are evaluated two velocities at a time,
-// paired so that each pair is also a pair of the six face fluxes; the values are
-// those of the scalar routine with its products and sums contracted to FMAs.
+// Interface distribution on a face between cell L (below/left) and R (above/right), along
+// axis AX (0: face of constant x, 1: of constant y), from the staged fbar+ of the two
+// cells and their neighbours, and (xi . n_+ l) f_b of the six crossing velocities (n_+ = +x or +y)
+// from it.  Paired arithmetic: on this GPU one FFMA2/FMUL2 instruction does two independent FP32
+// operations (each rounded as the scalar operation), so the reconstructions are evaluated two
+// velocities at a time, paired so that each pair is also a pair of the six face fluxes.
 __device__ __forceinline__ float2 p2(float a, float b) { return make_float2(a, b); }
 
 // fbar+ of velocity plane a at l plus cx (E - W) [plus cy (N - S)], for two
@@ -529,20 +483,15 @@ __device__ __forceinline__ void cart_tile(const CartInst &m, int par, int tbx, i
             for (int a = 0; a < NQ; a++)
                 if constexpr (P == P_BF16DEV || P == P_FP16DEV) fv[a] += fe[a];       // decode the deviation
             if (mir == 0) {
-                if constexpr (P == P_FP64) {
+                // paired: a f + b feq for the velocity pairs (1,2) (3,4) (5,6) (7,8)
+                const float2 kb2 = make_float2(k.b, k.b), ka2 = make_float2(k.a, k.a);
+                s_fbp[ls] = k.a * fv[0] + k.b * fe[0];
 #pragma unroll
-                    for (int a = 0; a < NQ; a++) s_fbp[a * LXY + ls] = k.a * fv[a] + k.b * fe[a];
-                } else {
-                    // paired: a f + b feq for the velocity pairs (1,2) (3,4) (5,6) (7,8)
-                    const float2 kb2 = make_float2(k.b, k.b), ka2 = make_float2(k.a, k.a);
-                    s_fbp[ls] = k.a * fv[0] + k.b * fe[0];
-#pragma unroll
-                    for (int a = 1; a < NQ; a += 2) {
-                        const float2 v = __ffma2_rn(ka2, make_float2(fv[a], fv[a + 1]),
-                                                    __fmul2_rn(kb2, make_float2(fe[a], fe[a + 1])));
-                        s_fbp[a * LXY + ls] = v.x;
-                        s_fbp[(a + 1) * LXY + ls] = v.y;
-                    }
+                for (int a = 1; a < NQ; a += 2) {
+                    const float2 v = __ffma2_rn(ka2, make_float2(fv[a], fv[a + 1]),
+                                                __fmul2_rn(kb2, make_float2(fe[a], fe[a + 1])));
+                    s_fbp[a * LXY + ls] = v.x;
+                    s_fbp[(a + 1) * LXY + ls] = v.y;
                 }
             } else {
                 // mirror ghost: fbar+ of the mirrored velocity
@@ -571,8 +520,7 @@ __device__ __forceinline__ void cart_tile(const CartInst &m, int par, int tbx, i
         if (has_x(x0 + fi - 1) && has_x(x0 + fi) && has_y(y0 + fj)) {
             const int lL = (fj + 2) * S::SX + (fi + 1);
             R fl[6];
-            if constexpr (P == P_FP64) cart_interior_face<0, R>(fl, s_fbp, lL, lL + 1, sten(fi - 1, fj), sten(fi, fj), k, LXY);
-            else cart_interior_face_f32x2<0>(fl, s_fbp, lL, lL + 1, sten(fi - 1, fj), sten(fi, fj), k, LXY);
+            cart_interior_face_f32x2<0>(fl, s_fbp, lL, lL + 1, sten(fi - 1, fj), sten(fi, fj), k, LXY);
 #pragma unroll
             for (int r = 0; r < 6; r++) s_fx[r * S::NSX + slot] = fl[r];
         }
@@ -591,8 +539,7 @@ __device__ __forceinline__ void cart_tile(const CartInst &m, int par, int tbx, i
             if (has_y(y0 + fj - 1) && has_y(y0 + fj) && has_x(x0 + fi)) {
                 const int lB = (fj + 1) * S::SX + (fi + 2);
                 R fl[6];
-                if constexpr (P == P_FP64) cart_interior_face<1, R>(fl, s_fbp, lB, lB + S::SX, sten(fi, fj - 1), sten(fi, fj), k, LXY);
-                else cart_interior_face_f32x2<1>(fl, s_fbp, lB, lB + S::SX, sten(fi, fj - 1), sten(fi, fj), k, LXY);
+                cart_interior_face_f32x2<1>(fl, s_fbp, lB, lB + S::SX, sten(fi, fj - 1), sten(fi, fj), k, LXY);
 #pragma unroll
                 for (int r = 0; r < 6; r++) s_fy[r * S::NSY + qq] = fl[r];
             }
@@ -664,64 +611,35 @@ __device__ __forceinline__ void cart_tile(const CartInst &m, int par, int tbx, i
         }
 
         // ---- macroscopic flux -> W^{n+1} (FP64); cell update f^{n+1} (Eq. fn+1)
-        R M0 = R(0), M1 = R(0), M2 = R(0);
-        if constexpr (P == P_FP64) {
-#pragma unroll
-            for (int a = 0; a < NQ; a++) {
-                M0 += F[a];
-                if (EX(a) == 1) M1 += F[a]; else if (EX(a) == -1) M1 -= F[a];
-                if (EY(a) == 1) M2 += F[a]; else if (EY(a) == -1) M2 -= F[a];
-            }
-        } else {
-            // paired: sum xi_x F = (F1 - F3) + (F5 - F7) - (F6 - F8), sum xi_y F = (F2 - F4) + (F5 - F7) + (F6 - F8)
-            const float2 m1 = p2(-1.f, -1.f);
-            const float2 q1 = p2(F[1], F[2]), q3 = p2(F[3], F[4]), q5 = p2(F[5], F[6]), q7 = p2(F[7], F[8]);
-            const float2 sm = __fadd2_rn(__fadd2_rn(q1, q3), __fadd2_rn(q5, q7));
-            const float2 d13 = __ffma2_rn(q3, m1, q1), d57 = __ffma2_rn(q7, m1, q5);
-            M0 = F[0] + (sm.x + sm.y);
-            M1 = d13.x + (d57.x - d57.y);
-            M2 = d13.y + (d57.x + d57.y);
-        }
+        // paired: sum xi_x F = (F1 - F3) + (F5 - F7) - (F6 - F8), sum xi_y F = (F2 - F4) + (F5 - F7) + (F6 - F8)
+        const float2 m1 = p2(-1.f, -1.f);
+        const float2 q1 = p2(F[1], F[2]), q3 = p2(F[3], F[4]), q5 = p2(F[5], F[6]), q7 = p2(F[7], F[8]);
+        const float2 sm = __fadd2_rn(__fadd2_rn(q1, q3), __fadd2_rn(q5, q7));
+        const float2 d13 = __ffma2_rn(q3, m1, q1), d57 = __ffma2_rn(q7, m1, q5);
+        const R M0 = F[0] + (sm.x + sm.y), M1 = d13.x + (d57.x - d57.y), M2 = d13.y + (d57.x + d57.y);
         const R d0 = k.dtV * M0, d1 = k.dtV * M1, d2 = k.dtV * M2;
         const double W0 = w0n - to_f64<R>(d0), W1 = w1n - to_f64<R>(d1), W2 = w2n - to_f64<R>(d2);
-        // FP32 compute: the FP64 sums are stored last, after the f update, which does not
-        // wait for them (the FP64 unit of this GPU is narrow)
-        if constexpr (P == P_FP64) {
-            Wout[g] = W0;
-            Wout[np + g] = W1;
-            Wout[2 * np + g] = W2;
-        }
+        // the FP64 sums are stored last, after the f update, which does not wait for them (the
+        // FP64 unit of this GPU is narrow)
         R rho1, ux1, uy1, feq1[NQ];
-        if constexpr (P == P_FP64) {
-            rho1 = W0;
-            vel_of<R>(W0, W1, W2, ux1, uy1);
-            feq9f<R>(rho1, ux1, uy1, feq1);
-        } else {
-            const R drho1 = b0_n - d0;
-            rho1 = R(1) + drho1;
-            vel_of<R>(rho1, from_f64<R>(w1n) - d1, from_f64<R>(w2n) - d2, ux1, uy1);
-            feq9fd<R>(drho1, rho1, ux1, uy1, feq1);
-        }
-        if constexpr (P == P_FP64) {
+        const R drho1 = b0_n - d0;
+        rho1 = R(1) + drho1;
+        vel_of<R>(rho1, from_f64<R>(w1n) - d1, from_f64<R>(w2n) - d2, ux1, uy1);
+        feq9fd<R>(drho1, rho1, ux1, uy1, feq1);
+        // paired: (f - dt/V F + r feq) / (1 + r) for the velocity pairs
+        const float2 mdv = make_float2(-k.dtV, -k.dtV), r2 = make_float2(k.r, k.r);
+        const float2 i2 = make_float2(m.finv1r, m.finv1r);
+        fout[g] = SP::enc((fn[0] - k.dtV * F[0] + k.r * feq1[0]) * m.finv1r, feq1[0], 0);
 #pragma unroll
-            for (int a = 0; a < NQ; a++)
-                fout[a * np + g] = SP::enc((fn[a] - k.dtV * F[a] + k.r * feq1[a]) / (R(1) + k.r), feq1[a], a);
-        } else {
-            // paired: (f - dt/V F + r feq) / (1 + r) for the velocity pairs
-            const float2 mdv = make_float2(-k.dtV, -k.dtV), r2 = make_float2(k.r, k.r);
-            const float2 i2 = make_float2(m.finv1r, m.finv1r);
-            fout[g] = SP::enc((fn[0] - k.dtV * F[0] + k.r * feq1[0]) * m.finv1r, feq1[0], 0);
-#pragma unroll
-            for (int a = 1; a < NQ; a += 2) {
-                const float2 t = __ffma2_rn(mdv, make_float2(F[a], F[a + 1]), make_float2(fn[a], fn[a + 1]));
-                const float2 v = __fmul2_rn(__ffma2_rn(r2, make_float2(feq1[a], feq1[a + 1]), t), i2);
-                fout[a * np + g] = SP::enc(v.x, feq1[a], a);
-                fout[(a + 1) * np + g] = SP::enc(v.y, feq1[a + 1], a + 1);
-            }
-            Wout[g] = W0;
-            Wout[np + g] = W1;
-            Wout[2 * np + g] = W2;
+        for (int a = 1; a < NQ; a += 2) {
+            const float2 t = __ffma2_rn(mdv, make_float2(F[a], F[a + 1]), make_float2(fn[a], fn[a + 1]));
+            const float2 v = __fmul2_rn(__ffma2_rn(r2, make_float2(feq1[a], feq1[a + 1]), t), i2);
+            fout[a * np + g] = SP::enc(v.x, feq1[a], a);
+            fout[(a + 1) * np + g] = SP::enc(v.y, feq1[a + 1], a + 1);
         }
+        Wout[g] = W0;
+        Wout[np + g] = W1;
+        Wout[2 * np + g] = W2;
     }
 }
 
@@ -774,7 +692,7 @@ __device__ __forceinline__ bool cta_wait_staged(const CartInst &m, uint32_t bar,
 enum CartMode { CART_SPECIALISED = 0, CART_SPECIALISED_TMA = 1, CART_GENERAL = 2 };
 
 template <int P, int TX, int TY, int MODE, bool DIAG = false>
-__global__ void __launch_bounds__(cart_threads<TX, TY>(), P == P_FP64 ? 1 : (cart_threads<TX, TY>() <= 320 ? 4 : 2))
+__global__ void __launch_bounds__(cart_threads<TX, TY>(), cart_threads<TX, TY>() <= 320 ? 4 : 2)
 k_step_cart(const CartInst m, int par, const __grid_constant__ CUtensorMap tf, const __grid_constant__ CUtensorMap tw)
 {
     static_assert(!DIAG || MODE == CART_GENERAL, "diagnostic steps run every block on the general variant");
