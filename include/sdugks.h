@@ -194,7 +194,9 @@ int sdugks_step(sdugks_solver *s, int64_t n);
  * solver's units.  For a wall this is the force of the fluid on it, from which drag
  * and lift coefficients follow (C = F / (0.5 rho U^2 D), Sec. IV).  Periodic patches
  * read 0.  Synchronises.  The FP64 sums use atomics, so the last bits can vary from
- * run to run; the state update itself is unchanged. */
+ * run to run.  The state update is sdugks_step's, in FP64 to the bit; in FP32 a sum may
+ * be rounded differently (on Cartesian grids of many waves, whose ordinary steps run
+ * another form of the kernel). */
 int sdugks_step_forces(sdugks_solver *s, double *force);
 
 /* One step (as sdugks_step(s, 1)) that also returns the momentum leaving the fluid
