@@ -937,6 +937,7 @@ extern "C" int sdugks_solver_create(const sdugks_mesh *m, const sdugks_params *p
     // within a tile, cells along a Morton curve of their centroids (16 bits per axis over
     // the tile's bounding box): faces, which are listed in the order of their cells,
     // then read nearby local indices from one warp to the next lane
+    std::vector<std::pair<uint64_t, int32_t>> curve;
     for (const auto &t : final_tiles) {
         double mn[2] = {INFINITY, INFINITY}, mx[2] = {-INFINITY, -INFINITY};
         for (size_t i = t.first; i < t.second; i++)
@@ -955,10 +956,11 @@ extern "C" int sdugks_solver_create(const sdugks_mesh *m, const sdugks_params *p
             for (int b = 15; b >= 0; b--) k = (k << 2) | (((q[1] >> b) & 1u) << 1) | ((q[0] >> b) & 1u);
             return k;
         };
-        std::sort(ids.begin() + t.first, ids.begin() + t.second, [&](int32_t a, int32_t b) {
-            const uint64_t ka = key(a), kb = key(b);
-            return ka != kb ? ka < kb : a < b;
-        });
+        // (each key once: formed in every comparison, they took more than the rings of the halves below)
+        curve.clear();
+        for (size_t i = t.first; i < t.second; i++) curve.emplace_back(key(ids[i]), ids[i]);
+        std::sort(curve.begin(), curve.end());
+        for (size_t i = t.first; i < t.second; i++) ids[i] = curve[i - t.first].second;
     }
     // Small meshes, tile size left open: where twice the tiles still fit the device at once, the
     // step runs on half tiles (halves of the Morton curve, so the cell order, and with it a
