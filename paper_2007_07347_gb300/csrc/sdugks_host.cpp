@@ -2456,25 +2456,30 @@ static void fill_dvm_cart(DvmCart &k, const sdugks_mesh &m, const CartGrid &g, c
     // Sums over the nodes, every product and sum to twice double's precision and rounded once at
     // the end.  The steps use them over and over: added up one after another over the nv^2 nodes (errors
     // up to 5e-15) they put u off by 1.3e-13 after 200 steps of a 16 x 16 x 64^2 cavity in FP64.
-    // half: of t(x) x^p along one axis, over the nodes of one sign (the zero node of an odd grid in
-    // both halves, by half); whole: over both.
-    auto half = [&](const double *t, int pos, int pw) {
-        Two s;
+    // half[pos][p]: of t(x) x^p along one axis, over the nodes of one sign (the zero node of an odd grid
+    // in both halves, by half).
+    struct Axis {
+        Two half[2][5];
+        Two whole(int p) const { return half[0][p] + half[1][p]; }
+    };
+    auto sum_axis = [&](const double *t) {
+        Axis s;
         for (int j = 0; j < nv; j++) {
             const bool zero = nv % 2 && j == nv / 2;
-            if (!zero && (j >= nv / 2) != (pos != 0)) continue;
             Two v{(zero ? 0.5 : 1.0) * t[j], 0.0};
-            for (int q = 0; q < pw; q++) v = v * Two{x[j], 0.0};
-            s = s + v;
+            for (int p = 0; p < 5; p++) {
+                for (int pos = 0; pos < 2; pos++)
+                    if (zero || (j >= nv / 2) == (pos != 0)) s.half[pos][p] = s.half[pos][p] + v;
+                v = v * Two{x[j], 0.0};
+            }
         }
         return s;
     };
-    auto whole = [&](const double *t, int pw) { return half(t, 0, pw) + half(t, 1, pw); };
+    const Axis ref[2] = {sum_axis(m0.data()), sum_axis(m0.data() + nv)};
     for (int n = 0; n <= 4; n++)
-        for (int b = 0; b <= n; b++)
-            d.m0f[n * (n + 1) / 2 + b] = (whole(m0.data(), n - b) * whole(m0.data() + nv, b)).value();
+        for (int b = 0; b <= n; b++) d.m0f[n * (n + 1) / 2 + b] = (ref[0].whole(n - b) * ref[1].whole(b)).value();
     for (int q = 0; q < 2; q++)
-        for (int b = 0; b < 2; b++) d.m0s[q][b] = whole(m0.data() + q * nv, 2 * b).value();
+        for (int b = 0; b < 2; b++) d.m0s[q][b] = ref[q].whole(2 * b).value();
     // walls in the order E, W, N, S.  Over the velocities of sign `pos` along the wall's axis: sums of
     // xi_n times (1, x, y, (x^2 + y^2) / 2), each Maxwellian being a product of its factors.
     const int side_of[4] = {1, 3, 2, 0};
@@ -2486,19 +2491,18 @@ static void fill_dvm_cart(DvmCart &k, const sdugks_mesh &m, const CartGrid &g, c
         factors(t, moving ? m.bc_par[p][0] : 0.0, moving ? m.bc_par[p][1] : 0.0);
         const int ax = w >> 1;
         const Two sgn{w % 2 ? -1.0 : 1.0, 0.0}, bb{rnd(d.b), 0.0}, ob = Two{1.0, 0.0} + bb;
-        auto sums = [&](const double *tab, int pos, Two out[4]) {
-            const double *n = tab + ax * nv, *a = tab + (1 - ax) * nv;
-            const Two n1 = sgn * half(n, pos, 1), n2 = sgn * half(n, pos, 2), n3 = sgn * half(n, pos, 3);
-            const Two a0 = whole(a, 0), a1 = whole(a, 1), a2 = whole(a, 2);
-            out[0] = n1 * a0;
-            out[1 + ax] = n2 * a0;
-            out[2 - ax] = n1 * a1;
-            out[3] = Two{0.5, 0.0} * (n3 * a0 + n1 * a2);
+        auto sums = [&](const Axis &n, const Axis &a, int pos, Two out[4]) {       // along the normal, across
+            const Two n1 = sgn * n.half[pos][1], n2 = sgn * n.half[pos][2], n3 = sgn * n.half[pos][3];
+            out[0] = n1 * a.whole(0);
+            out[1 + ax] = n2 * a.whole(0);
+            out[2 - ax] = n1 * a.whole(1);
+            out[3] = Two{0.5, 0.0} * (n3 * a.whole(0) + n1 * a.whole(2));
         };
+        const Axis wx[2] = {sum_axis(t), sum_axis(t + nv)};
         Two go[4], gi[4], mo[4], mi[4];
         const int leaving = w % 2 ? 0 : 1;
-        sums(t, leaving, go); sums(t, 1 - leaving, gi);
-        sums(m0.data(), leaving, mo); sums(m0.data(), 1 - leaving, mi);
+        sums(wx[ax], wx[1 - ax], leaving, go); sums(wx[ax], wx[1 - ax], 1 - leaving, gi);
+        sums(ref[ax], ref[1 - ax], leaving, mo); sums(ref[ax], ref[1 - ax], 1 - leaving, mi);
         const Two minus{-1.0, 0.0};
         for (int q = 0; q < 4; q++) {
             const Two gq = bb * go[q] + ob * gi[q], rest = mo[q] + gq;
@@ -2538,67 +2542,6 @@ extern "C" int sdugks_dvm_create(const sdugks_mesh *m, const sdugks_dvm_params *
     const int64_t n = m->nc, nf = F.nf, Q = (int64_t)prm->nv * prm->nv;
     for (int64_t f = 0; f < nf; f++)
         if (F.own[f] == F.nbr[f]) return fail(SDUGKS_ERR_INVALID_MESH, "periodic pair joins a cell to itself");
-    {
-        // faces in the order of their first cell: the face kernel then writes the fluxes
-        // in cell order, and the cell kernel, which walks the cells backwards, first reads
-        // the fluxes written last (still in L2)
-        std::vector<int64_t> ord(nf);
-        std::iota(ord.begin(), ord.end(), int64_t(0));
-        std::stable_sort(ord.begin(), ord.end(), [&](int64_t a, int64_t b) { return F.own[a] < F.own[b]; });
-        Faces G;
-        G.nf = nf;
-        G.own.resize(nf); G.nbr.resize(nf); G.nl.resize(2 * nf); G.ro.resize(2 * nf); G.rk.resize(2 * nf);
-        for (int64_t i = 0; i < nf; i++) {
-            const int64_t f = ord[i];
-            G.own[i] = F.own[f]; G.nbr[i] = F.nbr[f];
-            for (int d = 0; d < 2; d++) {
-                G.nl[2 * i + d] = F.nl[2 * f + d]; G.ro[2 * i + d] = F.ro[2 * f + d]; G.rk[2 * i + d] = F.rk[2 * f + d];
-            }
-        }
-        F = std::move(G);
-    }
-
-    // cell slots in ascending merged face id; LLSR neighbours, offsets and inverse
-    std::vector<int32_t> cface((size_t)n * MAXF, -1), cnb((size_t)n * MAXF, -1);
-    std::vector<double> cd((size_t)n * MAXF * 2, 0.0), ainv((size_t)n * 3, 0.0), dtv(n);
-    std::vector<int> ns(n, 0);
-    for (int64_t f = 0; f < nf; f++)
-        for (int side = 0; side < 2; side++) {
-            const int64_t c = side == 0 ? F.own[f] : F.nbr[f];
-            if (c < 0) continue;
-            if (ns[c] >= MAXF) return fail(SDUGKS_ERR_INVALID_MESH, "cell %lld has more than %d faces", (long long)c, MAXF);
-            const int sl = ns[c]++;
-            cface[(size_t)c * MAXF + sl] = (int32_t)f | (side ? DVM_SECOND : 0);
-            const int64_t k = side == 0 ? F.nbr[f] : F.own[f];
-            if (k >= 0) {
-                cnb[(size_t)c * MAXF + sl] = (int32_t)k;
-                const double *rme = side == 0 ? &F.ro[2 * f] : &F.rk[2 * f];
-                const double *rot = side == 0 ? &F.rk[2 * f] : &F.ro[2 * f];
-                cd[((size_t)c * MAXF + sl) * 2] = rme[0] - rot[0];
-                cd[((size_t)c * MAXF + sl) * 2 + 1] = rme[1] - rot[1];
-            }
-        }
-    for (int64_t c = 0; c < n; c++) {
-        double axx = 0, axy = 0, ayy = 0;
-        for (int sl = 0; sl < MAXF; sl++) {
-            if (cnb[(size_t)c * MAXF + sl] < 0) continue;
-            const double dx = cd[((size_t)c * MAXF + sl) * 2], dy = cd[((size_t)c * MAXF + sl) * 2 + 1];
-            axx += dx * dx; axy += dx * dy; ayy += dy * dy;
-        }
-        const double det = axx * ayy - axy * axy, tr = axx + ayy;
-        if (det > 1e-14 * tr * tr) {
-            ainv[3 * c] = ayy / det; ainv[3 * c + 1] = -axy / det; ainv[3 * c + 2] = axx / det;
-        }
-        dtv[c] = prm->dt / m->vol[c];
-    }
-    std::vector<double> fgeo((size_t)nf * 6);
-    std::vector<int32_t> fown(nf), fnbr(nf);
-    for (int64_t f = 0; f < nf; f++) {
-        fown[f] = (int32_t)F.own[f];
-        fnbr[f] = (int32_t)F.nbr[f];
-        const double g6[6] = {F.nl[2 * f], F.nl[2 * f + 1], F.ro[2 * f], F.ro[2 * f + 1], F.rk[2 * f], F.rk[2 * f + 1]};
-        std::copy(g6, g6 + 6, &fgeo[(size_t)f * 6]);
-    }
     // velocity nodes: midpoints of a uniform nv x nv partition of [-vmax, vmax]^2; node
     // q = j + nv i (x fastest) is (vn[j], vn[i]) with weight h^2
     const double h = 2.0 * prm->vmax / prm->nv;
@@ -2608,6 +2551,73 @@ extern "C" int sdugks_dvm_create(const sdugks_mesh *m, const sdugks_dvm_params *
     // uniform Cartesian grids take their own step (k_dvm_cart.cu)
     CartGrid grid;
     const bool cart = prm->dt <= prm->tau && detect_cart(*m, grid) && dvm_cart_fits(prm->precision == SDUGKS_FP64 ? P_FP64 : P_FP32, n, prm->nv, grid.ny);
+    // (on which the general path's tables are not needed)
+    std::vector<int32_t> cface, cnb, fown, fnbr;
+    std::vector<double> cd, ainv, dtv, fgeo;
+    if (!cart) {
+        {
+            // faces in the order of their first cell: the face kernel then writes the fluxes
+            // in cell order, and the cell kernel, which walks the cells backwards, first reads
+            // the fluxes written last (still in L2)
+            std::vector<int64_t> ord(nf);
+            std::iota(ord.begin(), ord.end(), int64_t(0));
+            std::stable_sort(ord.begin(), ord.end(), [&](int64_t a, int64_t b) { return F.own[a] < F.own[b]; });
+            Faces G;
+            G.nf = nf;
+            G.own.resize(nf); G.nbr.resize(nf); G.nl.resize(2 * nf); G.ro.resize(2 * nf); G.rk.resize(2 * nf);
+            for (int64_t i = 0; i < nf; i++) {
+                const int64_t f = ord[i];
+                G.own[i] = F.own[f]; G.nbr[i] = F.nbr[f];
+                for (int d = 0; d < 2; d++) {
+                    G.nl[2 * i + d] = F.nl[2 * f + d]; G.ro[2 * i + d] = F.ro[2 * f + d]; G.rk[2 * i + d] = F.rk[2 * f + d];
+                }
+            }
+            F = std::move(G);
+        }
+
+        // cell slots in ascending merged face id; LLSR neighbours, offsets and inverse
+        cface.assign((size_t)n * MAXF, -1); cnb.assign((size_t)n * MAXF, -1);
+        cd.assign((size_t)n * MAXF * 2, 0.0); ainv.assign((size_t)n * 3, 0.0); dtv.resize(n);
+        std::vector<int> ns(n, 0);
+        for (int64_t f = 0; f < nf; f++)
+            for (int side = 0; side < 2; side++) {
+                const int64_t c = side == 0 ? F.own[f] : F.nbr[f];
+                if (c < 0) continue;
+                if (ns[c] >= MAXF) return fail(SDUGKS_ERR_INVALID_MESH, "cell %lld has more than %d faces", (long long)c, MAXF);
+                const int sl = ns[c]++;
+                cface[(size_t)c * MAXF + sl] = (int32_t)f | (side ? DVM_SECOND : 0);
+                const int64_t k = side == 0 ? F.nbr[f] : F.own[f];
+                if (k >= 0) {
+                    cnb[(size_t)c * MAXF + sl] = (int32_t)k;
+                    const double *rme = side == 0 ? &F.ro[2 * f] : &F.rk[2 * f];
+                    const double *rot = side == 0 ? &F.rk[2 * f] : &F.ro[2 * f];
+                    cd[((size_t)c * MAXF + sl) * 2] = rme[0] - rot[0];
+                    cd[((size_t)c * MAXF + sl) * 2 + 1] = rme[1] - rot[1];
+                }
+            }
+        for (int64_t c = 0; c < n; c++) {
+            double axx = 0, axy = 0, ayy = 0;
+            for (int sl = 0; sl < MAXF; sl++) {
+                if (cnb[(size_t)c * MAXF + sl] < 0) continue;
+                const double dx = cd[((size_t)c * MAXF + sl) * 2], dy = cd[((size_t)c * MAXF + sl) * 2 + 1];
+                axx += dx * dx; axy += dx * dy; ayy += dy * dy;
+            }
+            const double det = axx * ayy - axy * axy, tr = axx + ayy;
+            if (det > 1e-14 * tr * tr) {
+                ainv[3 * c] = ayy / det; ainv[3 * c + 1] = -axy / det; ainv[3 * c + 2] = axx / det;
+            }
+            dtv[c] = prm->dt / m->vol[c];
+        }
+        fgeo.resize((size_t)nf * 6);
+        fown.resize(nf); fnbr.resize(nf);
+        for (int64_t f = 0; f < nf; f++) {
+            fown[f] = (int32_t)F.own[f];
+            fnbr[f] = (int32_t)F.nbr[f];
+            const double g6[6] = {F.nl[2 * f], F.nl[2 * f + 1], F.ro[2 * f], F.ro[2 * f + 1], F.rk[2 * f], F.rk[2 * f + 1]};
+            std::copy(g6, g6 + 6, &fgeo[(size_t)f * 6]);
+        }
+    }
+
     DvmCart dc{};
     std::vector<double> m0, wt;
     std::vector<int32_t> nbt, at;
@@ -2696,7 +2706,7 @@ extern "C" int sdugks_dvm_create(const sdugks_mesh *m, const sdugks_dvm_params *
         const cudaError_t ee = cudaMemcpy(const_cast<void *>(dst), src, bytes, cudaMemcpyHostToDevice);
         if (ee != cudaSuccess && rc2 == SDUGKS_OK) rc2 = fail(SDUGKS_ERR_CUDA, "%s: %s", what, cudaGetErrorString(ee));
     };
-    const auto gcd = conv(cd), gai = conv(ainv), gfg = conv(fgeo), gvn = conv(vn);
+    const auto gvn = conv(vn);
     if (cart) {
         const auto gm0 = conv(m0), gwt = conv(wt);
         d->dc.nc = (int32_t)n; d->dc.nv = prm->nv; d->dc.Q = Q;
@@ -2715,6 +2725,7 @@ extern "C" int sdugks_dvm_create(const sdugks_mesh *m, const sdugks_dvm_params *
         *out = d;
         return SDUGKS_OK;
     }
+    const auto gcd = conv(cd), gai = conv(ainv), gfg = conv(fgeo);
     up(d->dm.cell_face, cface.data(), cface.size() * 4, "upload cell faces");
     up(d->dm.cell_nb, cnb.data(), cnb.size() * 4, "upload neighbours");
     up(d->dm.cell_d, gcd.data(), gcd.size(), "upload offsets");
