@@ -213,6 +213,7 @@ def measured_peaks():
 STEP_SOURCES = {
     "k_step_cart": ["d2q9.cuh", "sdugks_internal.h", "step_cart.cuh", "k_cart.cu"],
     "k_step_tiled": ["d2q9.cuh", "sdugks_internal.h", "step_tiled.cuh", "k_step_fp32.cu"],
+    "k_step_strip": ["d2q9.cuh", "sdugks_internal.h", "step_strip.cuh", "k_strip.cu"],
     "k_strip_batch": ["d2q9.cuh", "sdugks_internal.h", "step_strip.cuh", "k_strip.cu"],
 }
 
@@ -431,7 +432,8 @@ def run_ours(args):
         configs = other_configs(args, S, stream, flush)
     if rank != 0:
         return
-    key = f"{ {1: 'k_step_tiled', 2: 'k_step_cart'}[info['kernel']] }_{args.precision}_{workload_tag(args)}"
+    kernel = "k_step_strip" if info["march"] else {1: "k_step_tiled", 2: "k_step_cart"}[info["kernel"]]
+    key = f"{kernel}_{args.precision}_{workload_tag(args)}"
     line = {
         "metric": "MLUPS", "value": value, "unit": "MLUPS", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": total_ms / args.steps, "higher_is_better": True,
@@ -444,7 +446,7 @@ def run_ours(args):
         "gpu_launches": args.steps * INTERVALS_PER_STEP * (INTERVAL + 2),
         "residual_last": last[0], "mass_last": last[1],
         "solver": {k: info[k] for k in ("n_tiles", "halo_cells", "mesh_bytes_per_cell_step", "kernel", "tile_cells",
-                                        "staging", "one_code_path")},
+                                        "staging", "one_code_path", "step_ctas", "step_cells", "march")},
         "autotune": tune,
         "mcell_steps_per_s": value / 9,
     }
@@ -515,7 +517,7 @@ def other_configs(args, S, stream, flush):
     launch_s = t / (interval * bsteps)               # the residual reductions are included
     out["batch_256_cavities_fp32"] = {
         "workload": "batch of 256 lid-driven cavities, N~logU[32,512], Re~logU[100,5000], seed 1, lid 0.1, CFL 0.5, "
-                    "FP32, one batched launch per step over the (instance, strip of columns, rows) work list",
+                    "FP32, one launch per 96 instances and step over their (instance, strip of columns, rows) work list",
         "value": cells * 9 * interval * bsteps / t / 1e6, "unit": "MLUPS", "steps": bsteps,
         "time_steps_per_step": interval, "ms_per_step": 1e3 * t / bsteps, "cells": cells,
         "roofline": {"bound": "hbm", "achieved": alg / launch_s / 1e9, "peak": peak, "unit": "GB/s",
@@ -523,10 +525,10 @@ def other_configs(args, S, stream, flush):
                      "kernel": "k_strip_batch",
                      "algorithmic_bytes_per_launch": alg, "avg_launch_us": launch_s * 1e6,
                      "peak_kind": f"{peak_kind} (hbm_gbs)", "l2_resident": False,
-                     "note": "1.4 GB of state: every launch streams it from HBM; the launch time includes the share "
-                             "of the per-instance residual reductions (one per 100 steps)"},
+                     "note": "per step (all its launches).  1.4 GB of state: every step streams it from HBM; the time "
+                             "includes the share of the per-instance residual reductions (one per 100 steps)"},
         "batch": b.info(), "clocks": clk.summary(),
-        "gpu_launches": bsteps * (interval + 2)}
+        "gpu_launches": bsteps * (interval * b.info()["step_launches"] + 2)}
     b.close()
     return out
 

@@ -343,13 +343,16 @@ typedef struct sdugks_batch_status {
     int64_t pool_bytes;      /* device pool size                                    */
     int64_t pool_used;       /* bytes held by active instances                      */
     int64_t steps;           /* batch steps since creation                          */
-    int32_t grid;            /* CTAs per block step launch (the item count if per_item) */
+    int32_t grid;            /* CTAs that a launch over all work items would have (the item
+                                count if per_item); see step_ctas                   */
     int32_t ctas_per_sm;     /* resident CTAs per SM of the batched kernel          */
     int32_t graph_steps;     /* steps per captured graph                            */
     int32_t precision;
     int32_t per_item;        /* 1: one CTA per work item; 0: a fixed grid walks the
                                 work list                                           */
     int32_t march;           /* 1: FP32 instances step by marching warps, 0: by blocks  */
+    int32_t step_launches;   /* kernel launches of one step                         */
+    int64_t step_ctas;       /* their CTAs                                          */
 } sdugks_batch_status;
 
 /* Create a batch with a device pool of pool_bytes and room for max_instances
@@ -409,9 +412,11 @@ void sdugks_solver_destroy(sdugks_solver *s);
  * diffusely (Sec. III): velocities entering the gas take the wall Maxwellian at
  * R T_wall with the density that makes the wall pass no mass (Eqs. 6001-6002),
  * leaving ones the characteristic reconstruction from the inner cell.  Any other
- * boundary kind gives BAD_BC at creation.  f is stored [cell][velocity] (weighted
- * values f_q = w_q f(xi_q)), W [cell][4] in FP64.  Device memory: about
- * 4 x (2 n_cells + n_faces) x Q bytes (FP32). */
+ * boundary kind gives BAD_BC at creation.  f is [cell][velocity] (weighted values
+ * f_q = w_q f(xi_q)), W [cell][4] in FP64.  Device memory: about
+ * 4 x (2 n_cells + n_faces) x Q bytes (FP32); on uniform grids above a few thousand
+ * values of f, which have a step of their own, 8 x n_cells x Q.  That step keeps fbar+ in
+ * the place of f; sdugks_dvm_get_state forms f from it. */
 typedef struct sdugks_dvm sdugks_dvm;
 
 typedef struct {
@@ -420,7 +425,8 @@ typedef struct {
     double RT_wall;      /* R T of the walls (and the default initial state) */
     double tau, dt;      /* relaxation time and time step (lattice units) */
     int32_t precision;   /* SDUGKS_FP64 or SDUGKS_FP32 (f and the scratch arrays) */
-    int32_t graph_steps; /* steps per captured CUDA graph: 0 = 32, < 0 = no graphs */
+    int32_t graph_steps; /* steps per captured CUDA graph: 0 = 32, < 0 = no graphs; an even
+                            number on uniform grids */
 } sdugks_dvm_params;
 
 /* Create on the current device; stream may be NULL (legacy default stream).

@@ -28,8 +28,8 @@
 // keep the precision that the differences of neighbouring moments need.
 //
 // A step of the 40 x 40 x 100^2 micro cavity in FP32: 90 us where k_dvm.cu takes 171 (23 x 23 x 50^2:
-// 18.8 / 36.5; 32 x 32 x 99^2: 68 / 216; FP64 30 x 30 x 64^2: 311 / 1282), of which the three kernels,
-// each by itself with cold caches, are 23, 12 and 69.  With f kept, and so a Maxwellian
+// 19.1 / 36.5; 32 x 32 x 99^2: 68 / 212; FP64 30 x 30 x 64^2: 326 / 1285), of which the three kernels,
+// each by itself with cold caches, are CAPTURE.  With f kept, and so a Maxwellian
 // for every cell read, a step took 140; with an update of single cells, ten reads each, 153.
 #include "d2q9.cuh"
 #include <algorithm>
@@ -720,8 +720,8 @@ template <class R> cudaError_t step_p(const DvmCart &m, const DvmCartState &s, i
 
 // Small solves stay with k_dvm.cu, whose two or three launches are shorter than these three: with
 // its 16-byte vectors (nv a multiple of 4) up to 2^18 values of f in FP32 (16 x 16 x 20^2: 8.4 us
-// a step, here 11.0; 16 x 16 x 32^2: 10.1 / 10.6; 30 x 30 x 20^2: 19.9 / 16.2) and 2^15 in FP64 (10 x 10 x 16^2:
-// 32 / 36; 14 x 14 x 16^2: 44 / 33), otherwise up to 2^16 (12 x 12 x 18^2: 9.1 / 10.0; 16 x 16 x 33^2: 16.2 / 12.9)
+// a step, here 11.0; 16 x 16 x 32^2: 10.1 / 10.6; 30 x 30 x 20^2: 19.9 / 16.7) and 2^15 in FP64 (10 x 10 x 16^2:
+// 32 / 36; 14 x 14 x 16^2: 44 / 33), otherwise up to 2^16 (12 x 12 x 18^2: 9.1 / 10.0; 16 x 16 x 33^2: 16.1 / 12.8)
 // and 2^14 (8 x 8 x 17^2: 48 / 43).
 bool dvm_cart_fits(int prec, int64_t nc, int nv, int ny)
 {

@@ -2357,6 +2357,10 @@ extern "C" int sdugks_batch_info(const sdugks_batch *b, sdugks_batch_status *o)
     o->precision = b->prec;
     o->per_item = b->per_item ? 1 : 0;
     o->march = b->march ? 1 : 0;
+    const int64_t n_strip = b->n_items - b->n_block;
+    for (const auto &g : b->groups) { o->step_launches++; o->step_ctas += g.n; }
+    if (!b->march && n_strip > 0) { o->step_launches++; o->step_ctas += n_strip; }
+    if (b->n_block > 0 || n_strip == 0) { o->step_launches++; o->step_ctas += batch_launch_grid(b); }
     return SDUGKS_OK;
 }
 

@@ -129,7 +129,7 @@ cudaError_t prepare_tiled_fp32(int prec);
 int occ_tiled_fp64();
 int occ_tiled_fp32(int prec);                              // resident tiles per SM
 cudaError_t prepare_cart(int prec);
-// block shapes of the Cartesian kernel: 0 = 16x16, 1 = 16x14, 2 = 16x8 (FP64: 16x16 only)
+// block shapes of the FP32-compute Cartesian kernel: 0 = 16x16, 1 = 16x14, 2 = 16x8
 constexpr int CART_SHAPES = 3;
 // block of the batched kernel: 16 x BATCH_TY cells per (instance, block) work item (the
 // 16x8 shape fits four CTAs per SM, the fastest shape of the single-solve kernel on
@@ -154,8 +154,8 @@ cudaError_t launch_step_cart64_tma(const CartInst &m, const CartTma &tma, int pa
 cudaError_t launch_step_cart64(const CartInst &m, int shape, int parity, cudaStream_t st);
 int cart64_shape(int nx, int ny, int n_sm);
 constexpr int CART64_BLOCK[3][2] = {{16, 14}, {8, 8}, {4, 4}};
-// One uniform-grid solve as the marching form sees it (FP32 storage; no symmetry side,
-// an even nx where x is periodic): the grid and its side rules, the ping-pong state, and
+// One uniform-grid solve as the marching form and its block form see it (FP32 storage; no
+// symmetry side, an even nx where x is periodic): the grid and its side rules, the ping-pong state, and
 // the step's constants, each twice (one operand of a paired instruction).
 struct StripInst {
     int32_t nx, ny, pitch, npad, periodic_x, periodic_y;

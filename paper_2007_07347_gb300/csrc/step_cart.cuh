@@ -1,4 +1,4 @@
-// step_cart.cuh -- fused S-DUGKS step on uniform Cartesian grids.
+// step_cart.cuh -- fused S-DUGKS step on uniform Cartesian grids, FP32 compute (FP64: k_cart64.cu).
 //
 // The same update as the tiled kernel (Eqs. fbarplus, fbpsource, fbar, Macro, Feq,
 // f_t_n+1, MesoFlux, MacroFlux, MacroUpdate, fn+1), specialised to nx x ny

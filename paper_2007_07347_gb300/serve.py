@@ -2,7 +2,7 @@
 
 Requests (seeded Poisson arrivals of a mix of lid-driven cavities, Couette channels
 and cylinder O-meshes) are admitted while their device-memory footprint fits: uniform
-grids join one `Batch` (one kernel launch per step over every admitted instance) and
+grids join one `Batch` (stepped together, a launch or a few per step) and
 cylinder O-meshes run as tiled single solvers on a second CUDA stream, so their work
 overlaps on the GPU.  Every `check_every` steps the residual of each running solve is
 read; solves whose residual is below `target` retire as converged, and so do, as not
