@@ -61,11 +61,11 @@ int strip_count(int nx, bool periodic_x)
     return nx <= STRIP_W ? 1 : (nx - (STRIP_W - STRIP_STEP) + STRIP_STEP - 1) / STRIP_STEP;
 }
 
-// Coefficients that share one whole (a + b = 1, 1/(1 + r) + r/(1 + r) = 1, c + b c = 1 times a
-// face's length and dt/V), for every cell and step the same: where each is rounded by itself, the
-// whole is off by up to 1e-7, alike in every step.  The larger part is rounded and the smaller one
-// is what it leaves of the whole (448^2, 300 steps: u off by 1.7e-7 with the former, 0.8e-7 with
-// the latter, 1.1e-7 by blocks; 8 cavities of 32^2 to 128^2, 500 steps: 4.2e-6, 0.9e-6, 3.2e-6).
+// The parts of one whole (a face's c + b c = 1 times its length and dt/V), for every cell and step the same:
+// rounded each by itself, and from rounded factors, the whole is off by up to 1e-7, alike in every
+// step.  The larger part is rounded and the smaller one is what it leaves of the whole (448^2, 300 steps, with
+// the same for a + b and 1/(1+r) + r/(1+r), which the step has as 1 - b and 1 - r/(1+r): u off by 1.7e-7
+// before, 0.8e-7 now, 1.1e-7 by blocks; 8 cavities of 32^2 to 128^2, 500 steps: 4.2e-6, 0.9e-6, 3.2e-6).
 static float part_of(double part, double whole)
 {
     return part > 0.5 * whole ? (float)part : (float)(whole - (double)(float)(whole - part));
@@ -87,9 +87,7 @@ void fill_strip(const CartInst &m, StripInst &s)
         s.side_drho[k] = m.fside_drho[k];
     }
     for (int b = 0; b < 2; b++) { s.f[b] = static_cast<float *>(m.f[b]); s.W[b] = m.W[b]; }
-    s.a = two(whole_less(m.b, 1.0)); s.b = two(part_of(m.b, 1.0));
-    const double ri = m.r / (1.0 + m.r);
-    s.inv = two(whole_less(ri, 1.0)); s.ri = two(part_of(ri, 1.0));
+    s.b = two((float)m.b); s.ri = two((float)(m.r / (1.0 + m.r)));
     s.sc = (float)(1.0 / (1.0 + m.b)); s.sb = (float)(1.0 / (double)s.sc - 1.0);
     for (int x = 0; x < 2; x++) {
         const double lv = (x == 0 ? m.dy : m.dx) * m.dtV, bg = lv * m.b / (1.0 + m.b);

@@ -164,7 +164,7 @@ struct StripInst {
     float sb, sc, len_dtV[2];                  // b, c; lengths of faces of constant x, y times dt / V
     float *f[2];
     double *W[2];
-    float2 a, b, inv, ri;                      // inv = 1 / (1 + r), ri = r inv
+    float2 b, ri;                              // ri = r / (1 + r)
     float2 g[2], bg[2];                        // faces of constant x, y: c len dt/V, b c len dt/V
     float2 xdt[2], xh[2], xo[2];               // dt, h/2, h/2 - dt along x, times 1/(2 dx); [1] negated
     float2 ydt[2], yh[2], yo[2];

@@ -14,8 +14,8 @@
 // for every face, and waits at two barriers per block: 1,169 thread instructions per cell.
 // Here the ring is four columns in 64 and four rows per range, each difference is formed
 // once per cell, both cells of a lane go through the same paired FP32 instructions
-// (FFMA2/FMUL2/FADD2), and the equilibria come scaled by the factor they are used with:
-// 420 per cell (1024^2, 16 rows per warp).  Measured (GB300, FP32 cavity, us per step,
+// (FFMA2/FMUL2/FADD2), and the faces' equilibria come scaled by the factor they are used with:
+// 440 per cell (1024^2, 16 rows per warp).  Measured (GB300, FP32 cavity, us per step,
 // blocks -> strips): 512^2 14.0 -> 11.3, 723^2 24.1 -> 19.8, 1024^2 48.8 -> 34.2, 2048^2
 // 181 -> 112 (4.5 TB/s of the state's bytes).
 //
@@ -26,6 +26,13 @@
 // saturates), three rows per loop turn without register moves (the code outgrows the
 // instruction cache: 34 % slower), a three-row ring (the copies are then only half a row
 // ahead), the flux sums in shared memory (3 % slower).
+//
+// fbar+ = f + b (feq - f) and f^{n+1} = t + r/(1+r) (feq - t), t = f - flux sum, take the equilibrium unscaled
+// and by the same operations: the rounding of feq that f took over then cancels in feq - f.  With the
+// equilibria scaled by b and by r/(1+r), each rounded its own way, what they differ by was multiplied by b
+// = dt/(2 tau), 10 to 100 on small grids at high Re: the FP32 residual's floor was 1.3 to 2.4 times
+// that of the blocks (48^2, Re 1000: 6.0e-7; blocks 3.6e-7, now 3.1e-7), and 4 of 100 served solves no
+// longer reached 1e-6.
 #pragma once
 #include "step_cart.cuh"
 
@@ -179,11 +186,11 @@ __device__ __forceinline__ void strip_update(const float2 F[NQ], const StripInst
     const float2 drho1 = sub2(b0, d[0]), rho1 = __fadd2_rn(dup(1.0f), drho1), inv = rcp2(rho1);
     const float2 ux1 = __fmul2_rn(sub2(m1, d[1]), inv), uy1 = __fmul2_rn(sub2(m2, d[2]), inv);
     float2 fe[NQ], v[NQ];
-    feq_pair(__fmul2_rn(m.ri, drho1), __fmul2_rn(m.ri, rho1), ux1, uy1, fe);
+    feq_pair(drho1, rho1, ux1, uy1, fe);
 #pragma unroll
     for (int a = 0; a < NQ; a++) {
-        const float2 fn = f(a);
-        v[a] = __ffma2_rn(m.inv, a == 0 ? fn : sub2(fn, F[a]), fe[a]);
+        const float2 fn = f(a), t = a == 0 ? fn : sub2(fn, F[a]);
+        v[a] = __ffma2_rn(m.ri, sub2(fe[a], t), t);
     }
     put_f(v);
 }
@@ -310,9 +317,12 @@ __device__ __forceinline__ void strip_march(const StripInst &m, int par, int xb,
         float2 b0, rho, ux, uy;
         state(slot, b0, rho, ux, uy);
         float2 fe[NQ];
-        feq_pair(__fmul2_rn(m.b, b0), __fmul2_rn(m.b, rho), ux, uy, fe);
+        feq_pair(b0, rho, ux, uy, fe);
 #pragma unroll
-        for (int a = 0; a < NQ; a++) out[a] = __ffma2_rn(m.a, row_f(slot, a), fe[a]);
+        for (int a = 0; a < NQ; a++) {
+            const float2 f = row_f(slot, a);
+            out[a] = __ffma2_rn(m.b, sub2(fe[a], f), f);
+        }
     };
 
     // next to a wall the one-sided difference takes the factor 1/h in the place of 1/(2h):

@@ -144,13 +144,13 @@ __device__ __forceinline__ void strip_block(StripBlockSmem &S, int par, int x0, 
             w0 = Wn[o]; w1 = Wn[o + np]; w2 = Wn[o + 2 * (int64_t)np];
 #pragma unroll
             for (int a = 0; a < NQ; a++) fn[a] = fin[o + (int64_t)np * a];
-            const float b0 = d2f_short(w0), rho = __fadd_rn(1.0f, b0), inv = recip<float>(rho), a = m.a.x, b = m.b.x;
-            feq_cell(__fmul_rn(b, b0), __fmul_rn(b, rho), __fmul_rn(d2f_short(w1), inv), __fmul_rn(d2f_short(w2), inv), e0, fe);
+            const float b0 = d2f_short(w0), rho = __fadd_rn(1.0f, b0), inv = recip<float>(rho), b = m.b.x;
+            feq_cell(b0, rho, __fmul_rn(d2f_short(w1), inv), __fmul_rn(d2f_short(w2), inv), e0, fe);
             float *const s = S.f + lj * SX + li;
-            s[0] = __fmaf_rn(a, fn[0], e0);
+            s[0] = __fmaf_rn(b, __fsub_rn(e0, fn[0]), fn[0]);
 #pragma unroll
             for (int k = 0; k < 4; k++) {
-                const float2 v = __ffma2_rn(dup(a), make_float2(fn[2 * k + 1], fn[2 * k + 2]), fe[k]);
+                const float2 f = make_float2(fn[2 * k + 1], fn[2 * k + 2]), v = __ffma2_rn(dup(b), sub2(fe[k], f), f);
                 s[(2 * k + 1) * PL] = v.x;
                 s[(2 * k + 2) * PL] = v.y;
             }
@@ -318,15 +318,16 @@ __device__ __forceinline__ void strip_block(StripBlockSmem &S, int par, int x0, 
     const float s2 = __fadd_rn(__fadd_rn(F[2], F[4]), __fadd_rn(F[6], F[8]));
     const float d0 = __fadd_rn(s1, s2), d1 = __fadd_rn(__fsub_rn(F[1], F[3]), __fsub_rn(d57, d68));
     const float d2 = __fadd_rn(__fsub_rn(F[2], F[4]), __fadd_rn(d57, d68));
-    const float drho = __fsub_rn(b0, d0), rho = __fadd_rn(1.0f, drho), inv = recip<float>(rho), ri = m.ri.x, i1 = m.inv.x;
+    const float drho = __fsub_rn(b0, d0), rho = __fadd_rn(1.0f, drho), inv = recip<float>(rho), ri = m.ri.x;
     float e0;
     float2 fe[4];
-    feq_cell(__fmul_rn(ri, drho), __fmul_rn(ri, rho), __fmul_rn(__fsub_rn(m1, d1), inv), __fmul_rn(__fsub_rn(m2, d2), inv), e0, fe);
+    feq_cell(drho, rho, __fmul_rn(__fsub_rn(m1, d1), inv), __fmul_rn(__fsub_rn(m2, d2), inv), e0, fe);
     float *const fo = m.f[1 - par] + o;
-    fo[0] = __fmaf_rn(i1, fn[0], e0);
+    fo[0] = __fmaf_rn(ri, __fsub_rn(e0, fn[0]), fn[0]);
 #pragma unroll
     for (int k = 0; k < 4; k++) {
-        const float2 v = __ffma2_rn(dup(i1), sub2(make_float2(fn[2 * k + 1], fn[2 * k + 2]), make_float2(F[2 * k + 1], F[2 * k + 2])), fe[k]);
+        const float2 t = sub2(make_float2(fn[2 * k + 1], fn[2 * k + 2]), make_float2(F[2 * k + 1], F[2 * k + 2]));
+        const float2 v = __ffma2_rn(dup(ri), sub2(fe[k], t), t);
         fo[(int64_t)np * (2 * k + 1)] = v.x;
         fo[(int64_t)np * (2 * k + 2)] = v.y;
     }
