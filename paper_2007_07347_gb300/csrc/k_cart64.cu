@@ -8,12 +8,17 @@
 // instruction holds its SM's pipe for 16 cycles, and a step costs the sum over the blocks
 // of an SM.  The form therefore spends as few FP64 instructions as it can: products are
 // contracted, the three divisions of a state become one Newton reciprocal, the division by
-// 1 + r a product, equilibria come scaled by the factor they are used with (weights, dt/V,
-// face length), the two sides of a tangential velocity are averaged before they are
+// 1 + r a product, the faces' equilibria come scaled by the factor they are used with
+// (weights, dt/V, face length), the two sides of a tangential velocity are averaged before they are
 // extrapolated, and beside a wall the missing neighbour is staged as the linear
 // extrapolation 2 f_0 - f_1, which makes the one-sided difference a central one and every
-// face of a block the same code.  About 380 FP64 warp instructions per 32 cells of a 16x14
-// block, where the earlier form took about 800.
+// face of a block the same code.  About 400 FP64 warp instructions per 32 cells of a 16x14
+// block, where the earlier form took about 800 (256^2: 56 us a step, where it took 129).
+//
+// fbar+ = f + b (feq - f) and f^{n+1} = t + r/(1+r) (feq - t), t = f less the flux sum, take the equilibrium
+// unscaled and by the same operations: the rounding of feq that f took over then cancels.  Scaled by b and by
+// r/(1+r) (54 us a step), what the two differ by was multiplied by b = dt/(2 tau): u of 256^2 at Re 5000 was
+// off by 2.5e-14 (the earlier form 1.7e-14, now 1.5e-14), of 48^2 at Re 4000 by 1.6e-13 (1.3e-13, 0.96e-13).
 //
 // Block shapes: 16x14 where that fills the SMs, 8x8 and 4x4 for smaller grids, whose few
 // blocks would leave most SMs' pipes idle (a 4 x 64 channel: 16 blocks of 4x4 in the place of
@@ -24,10 +29,9 @@
 namespace sdugks {
 namespace {
 
-// Coefficients (host-computed): equilibria scaled by b (fbar+), by the faces' b c l dt/V and
-// by r / (1 + r); reconstruction offsets times 1 / (2 h).
+// Coefficients (host-computed); reconstruction offsets times 1 / (2 h).
 struct Cart64K {
-    double a, b, inv, ri, dtV, rdtV;   // rdtV = 1 / dtV
+    double b, ri, dtV, rdtV;           // ri = r / (1 + r), rdtV = 1 / dtV
     double g[2], bg[2];                // faces of constant x, y: c l dt/V, b c l dt/V
     double lv[2], c;                   // l dt/V; c
     double xdt, xh, xo, ydt, yh, yo;   // dt, h/2, h/2 - dt along x and y, times 1/(2 h)
@@ -76,8 +80,8 @@ template <int BX, int BY> struct Shape64 {
     static constexpr int NT = BX >= 16 ? 256 : (BX >= 8 ? 192 : 64);
     static constexpr int CTAS = BX >= 16 ? 2 : (BX >= 8 ? 4 : 8);
     static constexpr size_t SMEM = sizeof(double) * (size_t)(NQ * LP + 6 * (NXF + NYF));
-    // FP64 warp instructions of a block (staging 45, face 94, cell 86): the cost model
-    static constexpr int COST = (LP + 31) / 32 * 45 + (XF + YF) / 32 * 94 + (BX * BY + 31) / 32 * 86;
+    // FP64 warp instructions of a block (staging 53, face 94, cell 94): the cost model
+    static constexpr int COST = (LP + 31) / 32 * 53 + (XF + YF) / 32 * 94 + (BX * BY + 31) / 32 * 94;
     static_assert(BX * BY <= NT, "one cell per thread");
 };
 
@@ -209,11 +213,11 @@ __device__ __forceinline__ void cart64_block(const CartInst &m, const Cart64K &k
 #pragma unroll
         for (int a = 0; a < NQ; a++) fv[a] = fs[a * ws];
         const double iv = recip64(w0);
-        feq64<true>(k.b * w0, w1 * iv, w2 * iv, fe);
+        feq64<true>(w0, w1 * iv, w2 * iv, fe);
 #pragma unroll
         for (int a = 0; a < NQ; a++) {
             const int d = mir == 0 ? a : (mir == 1 ? MIRROR_X(a) : (mir == 2 ? MIRROR_Y(a) : MIRROR_X(MIRROR_Y(a))));
-            s_f[d * LP + p] = fma(k.a, fv[a], fe[a]);
+            s_f[d * LP + p] = fma(k.b, fe[a] - fv[a], fv[a]);
         }
     }
     __syncthreads();
@@ -325,9 +329,12 @@ __device__ __forceinline__ void cart64_block(const CartInst &m, const Cart64K &k
     Wout[np + g] = W1;
     Wout[2 * np + g] = W2;
     const double iv = recip64(W0);
-    feq64<true>(k.ri * W0, W1 * iv, W2 * iv, fe);
+    feq64<true>(W0, W1 * iv, W2 * iv, fe);
 #pragma unroll
-    for (int a = 0; a < NQ; a++) fout[a * np + g] = fma(k.inv, a == 0 ? fn[a] : fn[a] - F[a], fe[a]);
+    for (int a = 0; a < NQ; a++) {
+        const double t = a == 0 ? fn[a] : fn[a] - F[a];
+        fout[a * np + g] = fma(k.ri, fe[a] - t, t);
+    }
 }
 
 template <int BX, int BY, bool DIAG>
@@ -373,14 +380,14 @@ k_step_cart64_tma(const CartInst m, const Cart64K k, int par, const __grid_const
 Cart64K coefs64(const CartInst &m)
 {
     Cart64K k;
-    // parts of one whole, the larger rounded and the smaller what it leaves: rounded each by itself the
-    // whole is off, alike in every step (45^2, 1000 steps: rho off by 1.8e-15 at most, now 0.7e-15)
+    // parts of one whole, the larger rounded and the smaller what it leaves: rounded each by itself
+    // the whole is off, alike in every step
     auto parts = [](double q, double whole, double &p, double &r) {      // q of the whole in r, the rest in p
         if (q > 0.5 * whole) { r = q; p = whole - q; }
         else { p = whole - q; r = whole - p; }
     };
-    parts(m.b, 1.0, k.a, k.b);
-    parts(m.r / (1.0 + m.r), 1.0, k.inv, k.ri);
+    k.b = m.b;
+    k.ri = m.r / (1.0 + m.r);
     k.c = 1.0 / (1.0 + k.b);
     k.dtV = m.dtV; k.rdtV = 1.0 / m.dtV;
     k.lv[0] = m.dy * m.dtV; k.lv[1] = m.dx * m.dtV;
@@ -396,7 +403,7 @@ template <int BX, int BY> cudaError_t launch64(const CartInst &m, int parity, cu
     using Sh = Shape64<BX, BY>;
     const dim3 grid((m.nx + BX - 1) / BX, (m.ny + BY - 1) / BY);
     // no early start: the blocks have to lie evenly on the SMs' FP64 pipes (256^2, in this kernel's
-    // first form: 62.8 us, with it 87.3; now 54)
+    // first form: 62.8 us, with it 87.3; then 54, now 56)
     if (m.force || m.bface)
         return launch_step_kernel(false, k_step_cart64<BX, BY, true>, grid, dim3(Sh::NT), Sh::SMEM, st, m, coefs64(m), parity);
     return launch_step_kernel(false, k_step_cart64<BX, BY, false>, grid, dim3(Sh::NT), Sh::SMEM, st, m, coefs64(m), parity);
