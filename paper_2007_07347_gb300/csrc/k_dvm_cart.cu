@@ -29,7 +29,7 @@
 //
 // A step of the 40 x 40 x 100^2 micro cavity in FP32: 90 us where k_dvm.cu takes 171 (23 x 23 x 50^2:
 // 19.1 / 36.5; 32 x 32 x 99^2: 68 / 212; FP64 30 x 30 x 64^2: 326 / 1285), of which the three kernels,
-// each by itself with cold caches, are CAPTURE.  With f kept, and so a Maxwellian
+// each by itself with cold caches, are 24, 15 and 68.  With f kept, and so a Maxwellian
 // for every cell read, a step took 140; with an update of single cells, ten reads each, 153.
 #include "d2q9.cuh"
 #include <algorithm>

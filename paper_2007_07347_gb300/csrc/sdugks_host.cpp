@@ -753,7 +753,7 @@ static int create_cart(const sdugks_mesh &m, const CartGrid &g, const sdugks_par
     // FP32 grids of many waves march (step_strip.cuh), unless a block is asked for by its size, where
     // the two models say that it is faster: 1.95 us per unit of strip_rows' cost against 54 ps per cell of the blocks'
     // (16x8, padding included).  GB300, FP32 cavity, blocks / marching in us per step: 384^2
-    // 8.1 / 9.8, 448^2 11.3 / 9.8, 512^2 14.0 / 11.3, 1024^2 48.8 / 34.2, 2048^2 181 / 112.
+    // 8.1 / 9.8, 448^2 11.3 / 10.2, 512^2 14.0 / 11.7, 1024^2 48.1 / 31.8, 2048^2 180 / 113.
     if (!use_tma && prm->tile_cells == 0 && !s->cart_general && strip_fits(s->ci, prec)) {
         const int strips = strip_count(g.nx, g.px);
         double cost = 0.0;
@@ -1983,10 +1983,10 @@ static int batch_upload_tables(sdugks_batch *b)
     b->n_items = (int64_t)items.size();
     // FP32 instances without a symmetry side or an odd wrap: marching warps, or their block form where
     // the whole list is too little work for those.  Measured (GB300, us per step of n x n cavities, marching /
-    // blocks): 1 of 32^2 4.4 / 2.7, 4 of 128^2 9.1 / 5.0, 1 of 256^2 8.3 / 5.0, 64 of 32^2 10.0 / 5.2, 32 of 64^2
-    // 8.1 / 8.3, 4 of 256^2 14.2 / 13.7, 1 of 512^2 11.9 / 13.5, 64 of 64^2 12.5 / 14.6, 8 of 256^2 22.6 / 25.3,
-    // 2 of 512^2 19.2 / 24.9.  A unit of strip_rows' cost takes 1.9 to 2.3 us, the more the narrower the grids (edge
-    // strips), blocks 1.9 us and 5.8 ns each.
+    // blocks): 1 of 32^2 4.5 / 2.7, 4 of 128^2 9.3 / 5.1, 1 of 256^2 8.5 / 5.0, 64 of 32^2 10.1 / 5.3, 32 of 64^2
+    // 8.3 / 8.4, 4 of 256^2 14.5 / 13.9, 1 of 512^2 12.1 / 13.8, 64 of 64^2 12.7 / 14.8, 8 of 256^2 23.0 / 25.8,
+    // 2 of 512^2 19.7 / 25.4, 128 of 64^2 25.3 / 27.5.  A unit of strip_rows' cost takes 1.9 to 2.3 us, the more the
+    // narrower the grids (edge strips), blocks 1.9 us and 5.8 ns each.
     std::vector<size_t> si;
     std::vector<StripInst> records;
     for (size_t q = 0; q < b->inst.size(); q++)

@@ -15,11 +15,11 @@
 // Here the ring is four columns in 64 and four rows per range, each difference is formed
 // once per cell, both cells of a lane go through the same paired FP32 instructions
 // (FFMA2/FMUL2/FADD2), and the faces' equilibria come scaled by the factor they are used with:
-// 440 per cell (1024^2, 16 rows per warp).  Measured (GB300, FP32 cavity, us per step,
-// blocks -> strips): 512^2 14.0 -> 11.3, 723^2 24.1 -> 19.8, 1024^2 48.8 -> 34.2, 2048^2
-// 181 -> 112 (4.5 TB/s of the state's bytes).
+// about 415 per cell (1024^2, 16 rows per warp).  Measured (GB300, FP32 cavity, us per step,
+// blocks -> strips): 512^2 14.0 -> 11.7, 723^2 23.7 -> 19.3, 1024^2 48.1 -> 31.8, 2048^2
+// 180 -> 113 (4.5 TB/s of the state's bytes).
 //
-// What bounds it now: latency.  Eight warps per SM (234 registers) issue in 45 % of the
+// What bounds it now: latency.  Eight warps per SM (226 registers) issue in 45 % of the
 // cycles; dependent FP32 pairs and the shared-memory/shuffle queue (which also carries the
 // six FP64 additions per row, 16 cycles each on this GPU's two FP64 lanes per SM) are the
 // stalls.  Measured without gain: twelve warps per SM at 168 registers (the queue then

@@ -11,8 +11,8 @@
 // one velocity of two cells), which halves each thread's chain.
 //
 // Measured (GB300, us per step of a batch, marching / this form / cart_tile's blocks): 1 cavity of 32^2
-// 4.4 / 2.7 / 3.0, 4 of 128^2 9.1 / 5.0 / 5.0, 1 of 256^2 8.3 / 5.0 / 5.0, 64 of 64^2 12.5 / 14.6 / 16.0, 256 of
-// 32^2 45.5 / 15.2 / 16.0.  Two columns per thread, as in the marching form, took 3.5 and 5.8 us in the place
+// 4.5 / 2.7 / 3.0, 4 of 128^2 9.3 / 5.1 / 5.0, 1 of 256^2 8.5 / 5.0 / 5.0, 64 of 64^2 12.7 / 14.8 / 16.0, 256 of
+// 32^2 36.4 / 15.4 / 16.0.  Two columns per thread, as in the marching form, took 3.5 and 5.8 us in the place
 // of 2.7 and 5.0 (1 of 32^2, of 256^2).  Bound by the latency of the phases, and on full lists by issue.
 #pragma once
 #include "step_strip.cuh"
